@@ -135,7 +135,7 @@ __device__ void finalize_stats(const Es1dFp64Bufs &b, int slot, int nblocks, dou
 template <int ORDER, int SCHEME>
 __global__ void __launch_bounds__(512) pass_c_kernel(Es1dConst c, Es1dFp64Bufs b, int par,
                                                      int prev_slot, int prev_nblocks) {
-  extern __shared__ double sm[];
+  extern __shared__ __align__(16) double sm[];
   double *Es = sm;
   double *Jt = sm + c.nc;
   __shared__ double red[33];
@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(512) pass_c_kernel(Es1dConst c, Es1dFp64Bufs b
 template <int ORDER, int SCHEME>
 __global__ void __launch_bounds__(512) pass_e_kernel(Es1dConst c, Es1dFp64Bufs b, int par,
                                                      int slot) {
-  extern __shared__ double sm[];
+  extern __shared__ __align__(16) double sm[];
   double *Es = sm;
   double *Eh = sm + c.nc;
   double *Jt = sm + 2 * c.nc;
@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(512) pass_e_kernel(Es1dConst c, Es1dFp64Bufs b
 template <int ORDER>
 __global__ void __launch_bounds__(512) deposit_initial_kernel(Es1dConst c, Es1dFp64Bufs b,
                                                               int par) {
-  extern __shared__ double sm[];
+  extern __shared__ __align__(16) double sm[];
   double *Jt = sm;
   for (int i = threadIdx.x; i < c.nc; i += blockDim.x) Jt[i] = 0.0;
   __syncthreads();
@@ -317,7 +317,7 @@ __global__ void finalize_kernel(Es1dFp64Bufs b, int slot, int nblocks) {
 template <int ORDER>
 __global__ void __launch_bounds__(512) charge_kernel(Es1dConst c, const double *x,
                                                      const double *w, double *rho) {
-  extern __shared__ double sm[];
+  extern __shared__ __align__(16) double sm[];
   double *Jt = sm;
   for (int i = threadIdx.x; i < c.nc; i += blockDim.x) Jt[i] = 0.0;
   __syncthreads();

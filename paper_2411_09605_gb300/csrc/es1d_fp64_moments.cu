@@ -111,7 +111,7 @@ struct MarkerE {
 template <int ORDER, int SCHEME, bool FOLD>
 __global__ void __launch_bounds__(512, 2) mom_pass_c_kernel(Es1dConst c, Es1dFp64Bufs b, int par,
                                                             int prev_slot) {
-  extern __shared__ double sm[];
+  extern __shared__ __align__(16) double sm[];
   __shared__ double red[kRedWords];
   const int nc = c.nc;
   const int nblk = (int)gridDim.x - 1;
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(512, 2) mom_pass_c_kernel(Es1dConst c, Es1dFp6
 template <int ORDER, int SCHEME, bool FOLD>
 __global__ void __launch_bounds__(512, 2) mom_pass_e_kernel(Es1dConst c, Es1dFp64Bufs b, int par,
                                                             int slot) {
-  extern __shared__ double sm[];
+  extern __shared__ __align__(16) double sm[];
   __shared__ double red[kRedWords];
   const int nc = c.nc;
   const int nblk = (int)gridDim.x - 1;
@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(512, 2) mom_absmax_kernel(Es1dConst c, Es1dFp6
 template <int ORDER>
 __global__ void __launch_bounds__(512, 2) mom_deposit_initial_kernel(Es1dConst c, Es1dFp64Bufs b,
                                                                      int par) {
-  extern __shared__ double sm[];
+  extern __shared__ __align__(16) double sm[];
   const int nc = c.nc;
   unsigned *T = (unsigned *)(sm + table_words<ORDER>(nc) + (nc + 1) / 2 * 2);
   const int copies = c.copies;

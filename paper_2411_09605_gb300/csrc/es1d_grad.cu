@@ -80,7 +80,7 @@ __device__ __forceinline__ double grid_mean(const Es1dConst &c, const double *a,
 // rev1: from the adjoints of x', v' to those of d, R and the deposit of H_bar.
 template <int ORDER>
 __global__ void __launch_bounds__(256) rev1_kernel(Es1dConst c, Es1dGradBufs g) {
-  extern __shared__ double tile[];
+  extern __shared__ __align__(16) double tile[];
   for (int i = threadIdx.x; i < c.nc; i += blockDim.x) tile[i] = 0.0;
   __syncthreads();
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < c.n_total;
@@ -142,7 +142,7 @@ __global__ void grid1_kernel(Es1dConst c, Es1dGradBufs g) {
 // rev2: J2_bar gathered at y -> adjoints of u, y and w; then through y, u, a.
 template <int ORDER>
 __global__ void __launch_bounds__(256) rev2_kernel(Es1dConst c, Es1dGradBufs g) {
-  extern __shared__ double tile[];
+  extern __shared__ __align__(16) double tile[];
   for (int i = threadIdx.x; i < c.nc; i += blockDim.x) tile[i] = 0.0;
   __syncthreads();
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < c.n_total;
@@ -236,7 +236,7 @@ __global__ void prep_kernel(Es1dConst c, Es1dGradBufs g, const double *E, const 
 // J1 = (q/h) sum w v S(x*) of the step's markers (ESEC2).
 template <int ORDER>
 __global__ void __launch_bounds__(256) dep_j1_kernel(Es1dConst c, Es1dGradBufs g) {
-  extern __shared__ double tile[];
+  extern __shared__ __align__(16) double tile[];
   for (int i = threadIdx.x; i < c.nc; i += blockDim.x) tile[i] = 0.0;
   __syncthreads();
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < c.n_total;
