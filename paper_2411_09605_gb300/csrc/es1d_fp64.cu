@@ -391,18 +391,14 @@ cudaError_t es1d_fp64_prepare(const Es1dConst &c) {
   dispatch(c.order, c.scheme, [&](auto O, auto S) {
     constexpr int ORDER = decltype(O)::value, SCHEME = decltype(S)::value;
     int smc = (int)(sizeof(double) * 2 * c.nc), sme = (int)(sizeof(double) * 3 * c.nc);
-    e = cudaFuncSetAttribute(pass_c_kernel<ORDER, SCHEME>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, smc);
+    e = allow_shared(pass_c_kernel<ORDER, SCHEME>, smc);
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(pass_e_kernel<ORDER, SCHEME>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, sme);
+      e = allow_shared(pass_e_kernel<ORDER, SCHEME>, sme);
     int sm1 = (int)(sizeof(double) * c.nc);
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(deposit_initial_kernel<ORDER>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, sm1);
+      e = allow_shared(deposit_initial_kernel<ORDER>, sm1);
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(charge_kernel<ORDER>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               sm1);
+      e = allow_shared(charge_kernel<ORDER>, sm1);
   });
   return e;
 }

@@ -373,7 +373,7 @@ cudaError_t es1d_mom_prepare(const Es1dConst &c) {
                           (const void *)mom_pass_e_kernel<ORDER, SCHEME, FOLD>,
                           (const void *)mom_deposit_initial_kernel<ORDER>})
       if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        e = allow_shared(k, most);
   });
   return e;
 }

@@ -287,7 +287,7 @@ cudaError_t es1d_grad_prepare(const Es1dConst &c) {
                  (const void *)rev1_kernel<1>, (const void *)rev1_kernel<2>,
                  (const void *)rev2_kernel<1>, (const void *)rev2_kernel<2>})
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+      e = allow_shared(k, sm);
   return e;
 }
 

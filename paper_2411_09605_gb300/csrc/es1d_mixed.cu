@@ -1553,27 +1553,21 @@ cudaError_t es1d_mix_prepare(const Es1dMixConst &c) {
     constexpr int ORDER = decltype(O)::value, SCHEME = decltype(S)::value;
     constexpr int MODE = decltype(M)::value, NT = decltype(RT)::value, NE = decltype(RE)::value;
     constexpr bool G64 = decltype(G)::value, FILT = decltype(F)::value;
-    e = cudaFuncSetAttribute(mix_pass_c_kernel<ORDER, SCHEME, MODE, NT, NE, FILT>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_c(c));
+    e = allow_shared(mix_pass_c_kernel<ORDER, SCHEME, MODE, NT, NE, FILT>, smem_c(c));
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(mix_pass_e_kernel<ORDER, SCHEME, MODE, NT, NE, G64, FILT>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_e(c));
+      e = allow_shared(mix_pass_e_kernel<ORDER, SCHEME, MODE, NT, NE, G64, FILT>, smem_e(c));
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(mix_deposit_initial_kernel<ORDER>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(8 * npad_host(c)));
+      e = allow_shared(mix_deposit_initial_kernel<ORDER>, 8 * npad_host(c));
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(mix_charge_kernel<ORDER>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(8 * npad_host(c)));
+      e = allow_shared(mix_charge_kernel<ORDER>, 8 * npad_host(c));
     if (e == cudaSuccess && c.wide == 1)
-      e = cudaFuncSetAttribute(mix_deposit_initial_wide_kernel<ORDER>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)(2 * 32 * 4 * npad_host(c)));
+      e = allow_shared(mix_deposit_initial_wide_kernel<ORDER>, 2 * 32 * 4 * npad_host(c));
   });
   if (e == cudaSuccess && c.scheme == 1 && c.mode == 0)
     dispatch_fused(c, [&](auto O, auto RT, auto RE, auto RE1) {
-      e = cudaFuncSetAttribute(mix_pass_ec_kernel<decltype(O)::value, decltype(RT)::value,
-                                                  decltype(RE)::value, decltype(RE1)::value>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_ec(c));
+      e = allow_shared(mix_pass_ec_kernel<decltype(O)::value, decltype(RT)::value,
+                                          decltype(RE)::value, decltype(RE1)::value>,
+                       smem_ec(c));
     });
   return e;
 }
@@ -1659,7 +1653,7 @@ cudaError_t es1d_batch_prepare(size_t smem, int threads) {
                              (const void *)mix_batch_pass_e_kernel<2, 256>};
   for (const void *k : threads == 1024 ? ks : ks_small)
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      e = allow_shared(k, smem);
   return e;
 }
 

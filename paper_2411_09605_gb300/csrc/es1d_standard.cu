@@ -274,12 +274,6 @@ void std_solve(const StdConst &c, const StdBufs &b, int slot, LaunchShape lp, cu
                    std_solve_smem(c), st, pdl, c, b, slot, lp.grid);
 }
 
-template <typename K>
-cudaError_t allow(K kernel, size_t bytes) {
-  if (bytes <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 }  // namespace
 
 LaunchShape std_shape(const StdConst &c, int nsm) {
@@ -297,9 +291,9 @@ cudaError_t std_prepare(const StdConst &c, const StdBufs &b, cudaStream_t st) {
   dispatch_std(c, [&](auto O, auto F) {
     constexpr int ORDER = decltype(O)::value;
     constexpr bool FOLD = decltype(F)::value;
-    if ((e = allow(std_step_kernel<ORDER, FOLD>, sm))) return;
-    if ((e = allow(std_charge_kernel<ORDER, FOLD>, sm))) return;
-    e = allow(std_solve_kernel, std_solve_smem(c));
+    if ((e = allow_shared(std_step_kernel<ORDER, FOLD>, sm))) return;
+    if ((e = allow_shared(std_charge_kernel<ORDER, FOLD>, sm))) return;
+    e = allow_shared(std_solve_kernel, std_solve_smem(c));
   });
   if (e != cudaSuccess) return e;
   std_response_kernel<<<(c.n + 3) / 4, 128, 0, st>>>(c, b);

@@ -427,6 +427,25 @@ struct LaunchShape {
   int block;
 };
 
+// Lets kern take `bytes` of dynamic shared memory, and with it all that a block can
+// have beside the kernel's static arrays: the attribute belongs to the kernel, so
+// that a limit at one handle's need would refuse the launches of another that needs
+// more, and without it the static arrays count against 48 KB too.
+template <typename K>
+cudaError_t allow_shared(K *kern, size_t bytes) {
+  int dev = 0, most = 0;
+  cudaFuncAttributes a;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, (const void *)kern);
+  if (e != cudaSuccess) return e;
+  const int room = most - (int)a.sharedSizeBytes;
+  if ((int64_t)bytes > room) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              room);
+}
+
 // Sets the message returned by pic_last_error (pic_api.cu).
 void set_last_error(const std::string &msg);
 
