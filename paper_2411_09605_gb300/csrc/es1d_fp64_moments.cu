@@ -353,7 +353,9 @@ size_t mom_smem(const Es1dConst &c) {
 // (its stencils are applied to whole tables) stays with the general passes.
 bool es1d_fp64_use_moments(const Es1dConst &c) { return c.nc <= kMomMaxNodes && c.passes == 0; }
 
-LaunchShape es1d_mom_shape(const Es1dConst &c, int nsm) { return fixed_shape(c.n_total, nsm, 1); }
+LaunchShape es1d_mom_shape(const Es1dConst &c, int nsm) {
+  return fixed_shape(c.n_total, nsm, 1, c.nc / 2);
+}
 
 int es1d_mom_copies(const Es1dConst &c, LaunchShape ls) {
   return fixed_copies((int64_t)c.nc * (c.order + 1), (c.n_total + ls.grid - 1) / ls.grid,

@@ -277,7 +277,7 @@ void std_solve(const StdConst &c, const StdBufs &b, int slot, LaunchShape lp, cu
 }  // namespace
 
 LaunchShape std_shape(const StdConst &c, int nsm) {
-  return fixed_shape(c.n_total, nsm, 0, std_smem(c, 1) <= kTwoBlockSmem ? 2 : 1);
+  return fixed_shape(c.n_total, nsm, 0, c.n / 2, std_smem(c, 1) <= kTwoBlockSmem ? 2 : 1);
 }
 int std_copies(const StdConst &c, LaunchShape ls) {
   return fixed_copies((int64_t)c.n * (c.order + 1), (c.n_total + ls.grid - 1) / ls.grid,

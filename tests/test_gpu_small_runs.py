@@ -1,0 +1,48 @@
+"""Times of small runs: a thousand markers take no longer than twenty thousand on
+the same grid.  Few markers leave a block the grid's own work (tables, tile, field
+solve), which a block sized by its markers alone gave to one warp: 2.2 to 3.9 times
+the time of the larger run."""
+import time
+
+import numpy as np
+import pytest
+
+from paper_2411_09605_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2411_09605_gb300 import build
+    build.build()
+
+
+def _step_seconds(sim):
+    sim.step(20)
+    best = np.inf
+    for _ in range(5):
+        t = time.perf_counter()
+        sim.step(100)
+        best = min(best, time.perf_counter() - t)
+    sim.close()
+    return best
+
+
+def _es(n):
+    from paper_2411_09605_gb300 import pic
+    return pic.Simulation(W.landau(n=n, nc=1792, order=2, dt=0.01, seed=1))
+
+
+def _spectral(n):
+    from paper_2411_09605_gb300 import pic
+    prob = W.weibel_1d2v(n=1024, ppc=20, order=2, dt=0.02, seed=1)
+    s = prob.species[0]
+    for k in ("y", "vx", "vy"):
+        setattr(s, k, np.ascontiguousarray(getattr(s, k)[:n]))
+    return pic.Simulation1D2V(prob)
+
+
+@pytest.mark.parametrize("make", [_es, _spectral])
+def test_fewer_markers_take_no_longer(make):
+    assert _step_seconds(make(1000)) <= 1.3 * _step_seconds(make(20_000))
