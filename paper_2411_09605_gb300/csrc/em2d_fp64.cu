@@ -1,6 +1,7 @@
 // 2D3V electromagnetic step with the leapfrog / Yee field update (Sec. 4.1,
-// Eq. EMleapfrog), FP64 form: the scheme, its charge-conserving option and what
-// both shapes' forms share (the point shapes run in em2d_fp64_moments.cu).
+// Eq. EMleapfrog), FP64 form: the scheme, its charge-conserving option, the point
+// shapes with few markers a cell (em2d_use_moments) and what both shapes' forms
+// share; other runs with point shapes take the passes of em2d_fp64_moments.cu.
 //
 // Yee lattice on a periodic nx x ny grid, component-major [3][ny][nx] arrays:
 //   Ex (i+1/2, j)  Ey (i, j+1/2)  Ez (i, j)      (J the same)
@@ -82,7 +83,39 @@ template <int OI, int OH>
 struct Shape2 {
   W1<OI> xI, yI;
   W1<OH> xH, yH;
+  static constexpr int kWeights = 2 * (OI + 1) + 2 * (OH + 1);
   Shape2() = default;
+  // the four axes' first nodes and weights, as store() wrote them for marker p
+  __device__ __forceinline__ void load(const double *sw, const int *si, int64_t p, int64_t n) {
+    xI.i0 = si[p];
+    xH.i0 = si[n + p];
+    yI.i0 = si[2 * n + p];
+    yH.i0 = si[3 * n + p];
+    int k = 0;
+#pragma unroll
+    for (int a = 0; a <= OI; a++) xI.w[a] = sw[(k++) * n + p];
+#pragma unroll
+    for (int a = 0; a <= OH; a++) xH.w[a] = sw[(k++) * n + p];
+#pragma unroll
+    for (int a = 0; a <= OI; a++) yI.w[a] = sw[(k++) * n + p];
+#pragma unroll
+    for (int a = 0; a <= OH; a++) yH.w[a] = sw[(k++) * n + p];
+  }
+  __device__ __forceinline__ void store(double *sw, int *si, int64_t p, int64_t n) const {
+    si[p] = xI.i0;
+    si[n + p] = xH.i0;
+    si[2 * n + p] = yI.i0;
+    si[3 * n + p] = yH.i0;
+    int k = 0;
+#pragma unroll
+    for (int a = 0; a <= OI; a++) sw[(k++) * n + p] = xI.w[a];
+#pragma unroll
+    for (int a = 0; a <= OH; a++) sw[(k++) * n + p] = xH.w[a];
+#pragma unroll
+    for (int a = 0; a <= OI; a++) sw[(k++) * n + p] = yI.w[a];
+#pragma unroll
+    for (int a = 0; a <= OH; a++) sw[(k++) * n + p] = yH.w[a];
+  }
   __device__ __forceinline__ Shape2(const Em2dConst &c, double x, double y) {
     const double xi = __dmul_rn(x, c.inv_hx), yi = __dmul_rn(y, c.inv_hy);
     xI.set(xi);
@@ -145,9 +178,13 @@ __device__ __forceinline__ void deposit_j(const Em2dConst &c, double *J, const S
   deposit_c<OI, OI>(J + 2 * nc, nx, ny, S.xI, S.yI, coef * u[2]);
 }
 
-// Shape orders of the charge-conserving form: the tent on integer-node axes, the
-// box on half-node axes.
-constexpr int kOrderI = 1, kOrderH = 0;
+// Shape orders of a form: the order on both axis kinds, or for the
+// charge-conserving form the tent on integer-node and the box on half-node axes
+template <int ORDER, bool CC>
+struct Orders {
+  static constexpr int I = CC ? 1 : ORDER;
+  static constexpr int H = CC ? 0 : ORDER;
+};
 
 // The pieces of the straight path from (x0, y0) by (dx, dy) between the grid
 // lines x = i hx and y = j hy, in path order: f(tau, xm, ym) with the piece's
@@ -270,29 +307,43 @@ __global__ void __launch_bounds__(256) em_k5_kernel(Em2dConst c, Em2dBufs b) {
   k5_block(c, b, blockIdx.x, gridDim.x, red);
 }
 
+template <int ORDER, bool CC>
 __global__ void __launch_bounds__(256) em_pass_c_kernel(Em2dConst c, Em2dBufs b) {
-  constexpr int OI = kOrderI, OH = kOrderH;
+  constexpr int OI = Orders<ORDER, CC>::I, OH = Orders<ORDER, CC>::H;
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < c.n_total;
        p += (int64_t)gridDim.x * blockDim.x) {
     const int s = species_of2(c, p);
     const double x = b.x[p], y = b.y[p];
     const double v[3] = {b.vx[p], b.vy[p], b.vz[p]};
     double vs[3], xh, yh;
-    const Shape2<OI, OH> Sx = shape_at_xstar<OI, OH>(c, b, x, y, v);
+    // ESEC2, point shapes: the shape at x* that the previous pass E (or the
+    // initial deposit) deposited j^{n,*} with, the same bits as forming it
+    Shape2<OI, OH> Sx;
+    if (!CC && b.sws)
+      Sx.load(b.sws, b.sis, p, c.n_total);
+    else
+      Sx = shape_at_xstar<OI, OH>(c, b, x, y, v);
     half_push_em<OI, OH>(c, b, s, Sx, x, y, v, vs, xh, yh);
     b.vsx[p] = vs[0];   // pass E forms x^{n+1/2} from v* with the same rounding
     b.vsy[p] = vs[1];
     b.vsz[p] = vs[2];
     const double coef = b.w ? c.q_a[s] * b.w[p] : c.qw_a[s];
-    for_pieces(c, x, y, c.dt * vs[0], c.dt * vs[1], b.err, [&](double tau, double xm, double ym) {
-      const Shape2<OI, OH> S(c, xm, ym);
-      deposit_j<OI, OH>(c, b.J2, S, coef * tau, vs);
-    });
+    if (CC) {
+      for_pieces(c, x, y, c.dt * vs[0], c.dt * vs[1], b.err, [&](double tau, double xm, double ym) {
+        const Shape2<OI, OH> S(c, xm, ym);
+        deposit_j<OI, OH>(c, b.J2, S, coef * tau, vs);
+      });
+    } else {
+      const Shape2<OI, OH> S(c, xh, yh);
+      deposit_j<OI, OH>(c, b.J2, S, coef, vs);
+      if (b.sw) S.store(b.sw, b.si, p, c.n_total);  // pass E gathers with it
+    }
   }
 }
 
+template <int ORDER, bool CC>
 __global__ void __launch_bounds__(256) em_pass_e_kernel(Em2dConst c, Em2dBufs b, int slot) {
-  constexpr int OI = kOrderI, OH = kOrderH;
+  constexpr int OI = Orders<ORDER, CC>::I, OH = Orders<ORDER, CC>::H;
   __shared__ double red[33];
   double ke = 0.0;
   unsigned nfb = 0;
@@ -302,20 +353,33 @@ __global__ void __launch_bounds__(256) em_pass_e_kernel(Em2dConst c, Em2dBufs b,
     const double x = b.x[p], y = b.y[p];
     const double v[3] = {b.vx[p], b.vy[p], b.vz[p]};
     const double vs[3] = {b.vsx[p], b.vsy[p], b.vsz[p]};
-    const double hdt = 0.5 * c.dt;   // x^{n+1/2} with pass C's rounding
-    const Shape2<OI, OH> S(c, wrapd(__fma_rn(hdt, vs[0], x), c.Lx, b.err),
-                           wrapd(__fma_rn(hdt, vs[1], y), c.Ly, b.err));
+    // the shape at x^{n+1/2} that pass C deposited with (point shapes, loaded:
+    // on this FP64-bound pass bytes are cheaper than its arithmetic), else
+    // formed again with pass C's rounding
+    Shape2<OI, OH> S;
+    if (!CC && b.sw) {
+      S.load(b.sw, b.si, p, c.n_total);
+    } else {
+      const double hdt = 0.5 * c.dt;
+      const double xh = wrapd(__fma_rn(hdt, vs[0], x), c.Lx, b.err);
+      const double yh = wrapd(__fma_rn(hdt, vs[1], y), c.Ly, b.err);
+      S = Shape2<OI, OH>(c, xh, yh);
+    }
     double e[3], bb[3];
-    // E^{n+1/2} over the path's pieces with the deposit's fractions and shapes
-    gather_eb<OI, OH>(c, nullptr, b.Bp, S, e, bb);
-    e[0] = e[1] = e[2] = 0.0;
-    for_pieces(c, x, y, c.dt * vs[0], c.dt * vs[1], b.err, [&](double tau, double xm, double ym) {
-      const Shape2<OI, OH> Sm(c, xm, ym);
-      double ek[3];
-      gather_eb<OI, OH>(c, b.Eh, nullptr, Sm, ek, nullptr);
+    if (CC) {
+      // E^{n+1/2} over the path's pieces with the deposit's fractions and shapes
+      gather_eb<OI, OH>(c, nullptr, b.Bp, S, e, bb);
+      e[0] = e[1] = e[2] = 0.0;
+      for_pieces(c, x, y, c.dt * vs[0], c.dt * vs[1], b.err, [&](double tau, double xm, double ym) {
+        const Shape2<OI, OH> Sm(c, xm, ym);
+        double ek[3];
+        gather_eb<OI, OH>(c, b.Eh, nullptr, Sm, ek, nullptr);
 #pragma unroll
-      for (int d = 0; d < 3; d++) e[d] += tau * ek[d];
-    });
+        for (int d = 0; d < 3; d++) e[d] += tau * ek[d];
+      });
+    } else {
+      gather_eb<OI, OH>(c, b.Eh, b.Bp, S, e, bb);
+    }
     const double k = c.dt * c.qm[s];
     const double vxb[3] = {vs[1] * bb[2] - vs[2] * bb[1], vs[2] * bb[0] - vs[0] * bb[2],
                            vs[0] * bb[1] - vs[1] * bb[0]};
@@ -342,6 +406,7 @@ __global__ void __launch_bounds__(256) em_pass_e_kernel(Em2dConst c, Em2dBufs b,
     if (c.scheme == 2) {
       const Shape2<OI, OH> S2 = shape_at_xstar<OI, OH>(c, b, xn, yn, vn);
       deposit_j<OI, OH>(c, b.J1, S2, b.w ? c.q_a[s] * wp : c.qw_a[s], vn);
+      if (!CC && b.sws) S2.store(b.sws, b.sis, p, c.n_total);  // the next pass C's
     }
     b.x[p] = xn;
     b.y[p] = yn;
@@ -357,14 +422,16 @@ __global__ void __launch_bounds__(256) em_pass_e_kernel(Em2dConst c, Em2dBufs b,
 }
 
 // j^{n,*} of the current state (start-up and after a state change)
+template <int ORDER, bool CC>
 __global__ void __launch_bounds__(256) em_deposit_initial_kernel(Em2dConst c, Em2dBufs b) {
-  constexpr int OI = kOrderI, OH = kOrderH;
+  constexpr int OI = Orders<ORDER, CC>::I, OH = Orders<ORDER, CC>::H;
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < c.n_total;
        p += (int64_t)gridDim.x * blockDim.x) {
     const int s = species_of2(c, p);
     const double v[3] = {b.vx[p], b.vy[p], b.vz[p]};
     const Shape2<OI, OH> S = shape_at_xstar<OI, OH>(c, b, b.x[p], b.y[p], v);
     deposit_j<OI, OH>(c, b.J1, S, b.w ? c.q_a[s] * b.w[p] : c.qw_a[s], v);
+    if (!CC && b.sws) S.store(b.sws, b.sis, p, c.n_total);  // pass C gathers with it
   }
 }
 
@@ -406,7 +473,12 @@ void em2d_k1(const Em2dConst &c, const Em2dBufs &b, LaunchShape lg, cudaStream_t
 }
 
 void em2d_pass_c(const Em2dConst &c, const Em2dBufs &b, LaunchShape lp, cudaStream_t st) {
-  em_pass_c_kernel<<<lp.grid, lp.block, 0, st>>>(c, b);
+  if (c.cc)
+    em_pass_c_kernel<1, true><<<lp.grid, lp.block, 0, st>>>(c, b);
+  else if (c.order == 1)
+    em_pass_c_kernel<1, false><<<lp.grid, lp.block, 0, st>>>(c, b);
+  else
+    em_pass_c_kernel<2, false><<<lp.grid, lp.block, 0, st>>>(c, b);
 }
 
 void em2d_k3(const Em2dConst &c, const Em2dBufs &b, LaunchShape lg, cudaStream_t st) {
@@ -415,7 +487,12 @@ void em2d_k3(const Em2dConst &c, const Em2dBufs &b, LaunchShape lg, cudaStream_t
 
 void em2d_pass_e(const Em2dConst &c, const Em2dBufs &b, int slot, LaunchShape lp,
                  cudaStream_t st) {
-  em_pass_e_kernel<<<lp.grid, lp.block, 0, st>>>(c, b, slot);
+  if (c.cc)
+    em_pass_e_kernel<1, true><<<lp.grid, lp.block, 0, st>>>(c, b, slot);
+  else if (c.order == 1)
+    em_pass_e_kernel<1, false><<<lp.grid, lp.block, 0, st>>>(c, b, slot);
+  else
+    em_pass_e_kernel<2, false><<<lp.grid, lp.block, 0, st>>>(c, b, slot);
 }
 
 void em2d_k5(const Em2dConst &c, const Em2dBufs &b, LaunchShape lg, cudaStream_t st, bool pdl) {
@@ -440,7 +517,12 @@ __global__ void em2d_validate_kernel(const double *x, const double *y, const dou
 
 void em2d_fp64_deposit_initial(const Em2dConst &c, const Em2dBufs &b, LaunchShape lp,
                                cudaStream_t st) {
-  em_deposit_initial_kernel<<<lp.grid, lp.block, 0, st>>>(c, b);
+  if (c.cc)
+    em_deposit_initial_kernel<1, true><<<lp.grid, lp.block, 0, st>>>(c, b);
+  else if (c.order == 1)
+    em_deposit_initial_kernel<1, false><<<lp.grid, lp.block, 0, st>>>(c, b);
+  else
+    em_deposit_initial_kernel<2, false><<<lp.grid, lp.block, 0, st>>>(c, b);
 }
 
 void em2d_fp64_bhalf(const Em2dConst &c, const double *B, const double *E, double *Bp,

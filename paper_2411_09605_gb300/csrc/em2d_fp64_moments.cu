@@ -1,5 +1,5 @@
-// The FP64 form's 2D3V Yee step with point shapes (em2d_fp64.cu states the scheme
-// and keeps the charge-conserving option), written to spare the FP64 pipe, which
+// The FP64 form's 2D3V Yee step with point shapes where a cell has markers enough
+// (em2d_use_moments; em2d_fp64.cu states the scheme and keeps the other runs), written to spare the FP64 pipe, which
 // bounds the marker passes (2 lanes per SM and clock):
 //
 //   gather    a component's B-spline interpolant in a cell is a polynomial of the
@@ -29,6 +29,7 @@
 // in shared memory, then the coefficients.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "em2d_common.cuh"
@@ -322,7 +323,7 @@ __global__ void __launch_bounds__(kPassThreads, 2) em_mom_c_kernel(Em2dConst c, 
   griddep_wait();
   const int64_t n = c.n_total, beg = blockIdx.x * c.chunk;
   const int64_t end = beg + c.chunk < n ? beg + c.chunk : n;
-  for (int64_t p0 = beg; p0 < end; p0 += kPassThreads) {   // whole warps: the deposits shuffle
+  for (int64_t p0 = beg; p0 < end; p0 += blockDim.x) {   // whole warps: the deposits shuffle
     const bool on = p0 + threadIdx.x < end;
     const int64_t p = p0 + threadIdx.x;   // lanes past the end work on zeros
     const int s = FOLD ? 0 : species_of2m(c, p);
@@ -382,7 +383,7 @@ __global__ void __launch_bounds__(kPassThreads, 2) em_mom_e_kernel(Em2dConst c, 
   const int64_t end = beg + c.chunk < n ? beg + c.chunk : n;
   double ke = 0.0;
   unsigned nfb = 0, bad = 0;
-  for (int64_t p0 = beg; p0 < end; p0 += kPassThreads) {
+  for (int64_t p0 = beg; p0 < end; p0 += blockDim.x) {
     const bool on = p0 + threadIdx.x < end;
     const int64_t p = p0 + threadIdx.x;   // lanes past the end work on zeros
     const int s = FOLD ? 0 : species_of2m(c, p);
@@ -461,7 +462,7 @@ template <int ORDER, bool FOLD>
 __global__ void __launch_bounds__(kPassThreads, 2) em_mom_start_kernel(Em2dConst c, Em2dBufs b) {
   const int64_t n = c.n_total, beg = blockIdx.x * c.chunk;
   const int64_t end = beg + c.chunk < n ? beg + c.chunk : n;
-  for (int64_t p0 = beg; p0 < end; p0 += kPassThreads) {
+  for (int64_t p0 = beg; p0 < end; p0 += blockDim.x) {
     const bool on = p0 + threadIdx.x < end;
     const int64_t p = p0 + threadIdx.x;   // lanes past the end work on zeros
     const int s = FOLD ? 0 : species_of2m(c, p);
@@ -507,11 +508,29 @@ void grid_launch(const Em2dConst &c, const Em2dBufs &b, int comps, cudaStream_t 
 
 }  // namespace
 
-// Two blocks of 256 per SM, each with an equal run of markers.
+// A marker costs less here (order 1: 0.31 ns of a step against 0.62, order 2: 0.56
+// against 0.98), a node more, 0.3 and 1.5 to 2 ns a step: its coefficients and
+// moments are 576 (order 2: 1296) bytes, written twice.  Order 1: a marker a node
+// pays for it, less some that the six launches' overlap pays for.  Order 2: five
+// markers a node, eleven where the coefficients (432 bytes a node) leave the L2, and
+// some more for launches that take longer; all runs on grids of up to 64 x 64.  us a
+// step (ESEC2), general passes / these: order 1, 1024 x 1024, 10^5 markers 248 / 542,
+// 2^21 markers 1406 / 1153; order 2, 256 x 256, 10^5 markers 162 / 267, 2^19 markers
+// 581 / 450; 1024 x 1024, 2^23 markers 8112 / 8691.
+bool em2d_use_moments(const Em2dConst &c) {
+  const int64_t nodes = (int64_t)c.nx * c.ny;
+  if (c.order == 1) return c.n_total + (1 << 14) >= nodes + nodes / 8;
+  return nodes <= 64 * 64 || c.n_total >= (nodes <= 1 << 18 ? 5 : 11) * nodes + 45'000;
+}
+
+// Two blocks of up to 256 per SM, each with an equal run of markers.  No warp is
+// without: one that is lets the next launch's blocks take the SMs before the others
+// are done (64 x 64, order 2, 57,344 markers: 135 us a step, with these 81).
 LaunchShape em2d_mom_shape(const Em2dConst &c, int nsm) {
   const int64_t most = 2 * (int64_t)nsm;
   const int64_t chunk = ((c.n_total + most - 1) / most + 31) / 32 * 32;
-  return LaunchShape{c.n_total ? (int)((c.n_total + chunk - 1) / chunk) : 1, kPassThreads};
+  return LaunchShape{c.n_total ? (int)((c.n_total + chunk - 1) / chunk) : 1,
+                     (int)std::min<int64_t>(kPassThreads, std::max<int64_t>(chunk, 32))};
 }
 int64_t em2d_mom_chunk(const Em2dConst &c, LaunchShape ls) { return fixed_chunk(c.n_total, ls); }
 

@@ -907,7 +907,7 @@ int restart_em2d(pic_handle *h, bool markers_changed = true) {
     CUDA_TRY(cudaMemsetAsync(mb.J2, 0, sizeof(long long) * nc3, h->st));
     if (h->ce.scheme == 2) em2dm_deposit_initial(h->cme, mb, h->lp, h->st);
   } else {
-    if (h->ce.cc) {
+    if (!h->ce.mom) {
       CUDA_TRY(cudaMemsetAsync(b.J1, 0, sizeof(double) * nc3, h->st));
       CUDA_TRY(cudaMemsetAsync(b.J2, 0, sizeof(double) * nc3, h->st));
       if (h->ce.scheme == 2) em2d_fp64_deposit_initial(h->ce, b, h->lp, h->st);
@@ -1048,7 +1048,9 @@ int init_em2d(pic_handle *h, const pic_species *species, const double *E0, const
   c.hdt = 0.5 * c.dt;
   for (int s = 0; s < h->nsp; s++) c.hdt_qm[s] = c.hdt * c.qm[s];
   c.fold = h->nsp == 1 && !h->weighted;
-  const bool mom = !h->mixed && !c.cc;   // the FP64 form with point shapes
+  const bool point = !h->mixed && !c.cc;   // the FP64 form with point shapes
+  const bool mom = point && em2d_use_moments(c);
+  c.mom = mom;
   if (mom)
     h->lp = em2d_mom_shape(c, h->nsm);
   else
@@ -1066,9 +1068,16 @@ int init_em2d(pic_handle *h, const pic_species *species, const double *E0, const
     return rc;
   // the moment passes hand the point x^{n+1/2} from pass C to pass E and, with
   // ESEC2, the next x* from pass E (or the initial deposit) to pass C
-  b.sd = b.sds = b.T = b.M1 = b.M2 = nullptr;
+  b.sw = b.sws = b.sd = b.sds = b.T = b.M1 = b.M2 = nullptr;
   b.si = b.sis = nullptr;
   const size_t words = (size_t)nc3 * (cfg.shape_order + 1) * (cfg.shape_order + 1);
+  // (the general ones: 4 first nodes and 4 (order + 1) weights a marker)
+  const size_t weights = (size_t)4 * (cfg.shape_order + 1) * h->N;
+  if (point && !mom &&
+      ((rc = h->alloc(&b.sw, weights)) || (rc = h->alloc(&b.si, (size_t)4 * h->N)) ||
+       (cfg.scheme == 2 &&
+        ((rc = h->alloc(&b.sws, weights)) || (rc = h->alloc(&b.sis, (size_t)4 * h->N))))))
+    return rc;
   if (mom && ((rc = h->alloc(&b.sd, (size_t)4 * h->N)) || (rc = h->alloc(&b.si, (size_t)2 * h->N)) ||
               (rc = h->alloc(&b.T, 2 * words)) || (rc = h->alloc(&b.M1, words)) ||
               (rc = h->alloc(&b.M2, words))))
@@ -1729,7 +1738,7 @@ int pic_step_async(pic_handle *h, int nsteps) {
       if (sort_now) swap_em2d_sorted(h);
       h->te_open = true;
       h->launches += 4;
-    } else if (!h->ce.cc) {
+    } else if (h->ce.mom) {
       CUDA_TRY(h->timed_launch(4, [&] { em2d_mom_k1(h->ce, e, h->st); }));
       CUDA_TRY(h->timed_launch(0, [&] { em2d_mom_pass_c(h->ce, e, h->lp, h->st); }));
       CUDA_TRY(h->timed_launch(4, [&] { em2d_mom_k3(h->ce, e, h->st); }));

@@ -171,6 +171,7 @@ struct Em2dConst {
   int nx, ny;
   int order;
   int cc;          // charge-conserving shapes and path pieces (order 1)
+  int mom;         // 1: the moment passes (FP64 form, em2d_use_moments)
   int scheme;
   int gamma_on;
   int nsp;
@@ -199,9 +200,12 @@ struct Em2dBufs {
   double *J1;     // j^{n,*}
   double *J2;     // j^{*,n+1/2}
   double *vsx, *vsy, *vsz;     // [N] v* of the current step (pass C -> pass E)
+  // general passes with point shapes (em2d_fp64.cu):
+  double *sw;     // [weights][N] shape at x^{n+1/2} (pass C -> pass E), si [4][N] its first nodes
+  double *sws;    // ESEC2: the shape at the next step's x*, with sis [4][N]
   // moment passes (em2d_fp64_moments.cu):
   double *sd;     // [4][N] offsets of x^{n+1/2} (dxI, dyI, dxH, dyH; pass C -> pass E)
-  int *si;        // [2][N] and its integer-node cells
+  int *si;        // [2][N] and its integer-node cells (null with sw and sd: formed again)
   double *sds;    // ESEC2: the next step's x* (pass E or the initial deposit -> pass C),
   int *sis;       // as sd / si; null: formed again
   double *T;      // [6 nc][(order + 1)^2] coefficients of E*, then E^{n+1/2}, and Bp
@@ -522,6 +526,7 @@ void es1d_fp64_kinetic(const Es1dConst &c, const double *v, const double *w, dou
                        cudaStream_t st);
 
 // 2D3V Yee path, FP64, point shapes (em2d_fp64_moments.cu)
+bool em2d_use_moments(const Em2dConst &c);
 LaunchShape em2d_mom_shape(const Em2dConst &c, int nsm);
 int64_t em2d_mom_chunk(const Em2dConst &c, LaunchShape ls);
 void em2d_mom_k1(const Em2dConst &c, const Em2dBufs &b, cudaStream_t st);

@@ -113,3 +113,12 @@ def test_yee_sizes(nx, ny, n, scheme, order):
         setattr(s, k, np.ascontiguousarray(getattr(s, k)[:n]))
     s.w0 = prob.Lx * prob.Ly / n
     yee._check(prob, scheme, steps=3)
+
+
+@pytest.mark.parametrize("scheme", [1, 2])
+@pytest.mark.parametrize("order,nx,ny,n", [(1, 150, 130, 5552), (1, 150, 130, 5553),
+                                           (2, 65, 64, 65_799), (2, 65, 64, 65_800)])
+def test_yee_line_between_the_passes(order, nx, ny, n, scheme):
+    """2D3V: the most markers that the general passes take on a grid and the fewest
+    of the moment passes."""
+    test_yee_sizes(nx, ny, n, scheme, order)
