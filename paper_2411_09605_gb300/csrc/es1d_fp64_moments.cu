@@ -17,7 +17,8 @@
 //             These are the B-spline weights of Sec. 2.2 term by term, so gather
 //             and deposit still use one shape and Eq. exp_econs_simple holds to
 //             rounding.
-//             The sums are exact integers (fixed_moments.cuh).
+//             The sums are exact integers, each node's with its own unit
+//             (fixed_moments.cuh).
 //   factors   of a single uniformly weighted species (FOLD) are not applied
 //             per marker: q w0 / h and m w0 / 2 go to the block's sums and dt q/m
 //             to the tables, so that pass C's gather is v* - v^n and pass
@@ -74,11 +75,20 @@ __device__ __forceinline__ void load_estar(const Es1dConst &c, const Es1dFp64Buf
 }
 
 // Shared memory of a pass: the table, F (nc values, the field the coefficients
-// are built from) and the tile copies (16-byte aligned: F padded to two words).
+// are built from), the tile copies (16-byte aligned: F padded to two words) and the
+// nodes' scale words.  On grids that those would cost the second block on an SM they
+// take F's place once the table is built (c.late, one more barrier).
 template <int ORDER>
-__device__ __forceinline__ size_t table_words(int nc) {
-  return (size_t)Poly<ORDER>::kWords * nc;
-}
+struct MomShared {
+  double *table, *F;
+  unsigned *T, *W;
+  __device__ __forceinline__ MomShared(const Es1dConst &c, double *sm) {
+    table = sm;
+    F = sm + (size_t)Poly<ORDER>::kWords * c.nc;
+    T = (unsigned *)(F + (c.nc + 1) / 2 * 2);
+    W = c.late ? (unsigned *)F : T + (size_t)2 * c.nc * (ORDER + 1) * c.copies;
+  }
+};
 
 // What a pass reads of marker p (nothing past the end).
 template <int SCHEME>
@@ -122,10 +132,17 @@ __global__ void __launch_bounds__(512, 2) mom_pass_c_kernel(Es1dConst c, Es1dFp6
       clear_doubles(b.J1[par ^ 1], nc);
       if (threadIdx.x == 0) b.Jt[par ^ 1] = 0.0;
     }
-    if (threadIdx.x == 0) b.amax[par ^ 1] = 0u;
-    if (prev_slot >= 0) {
-      double s = 0.0;
+    // where the next j^{n,*}'s largest amounts start (b.amax: [4][nc], J1 and J2 by parity)
+    const unsigned *e = b.amax + par * nc;
+    unsigned *next = b.amax + (par ^ 1) * nc;
+    const unsigned e0 = (int)threadIdx.x < nc ? __ldcg(e + threadIdx.x) : 0u;
+    double s = 0.0;
+    if (prev_slot >= 0)
       for (int i = threadIdx.x; i < nblk; i += blockDim.x) s += b.ke_part[i];
+    if ((int)threadIdx.x < nc) next[threadIdx.x] = scale_start(e0, c.decay);
+    for (int i = threadIdx.x + blockDim.x; i < nc; i += blockDim.x)
+      next[i] = scale_start(__ldcg(e + i), c.decay);
+    if (prev_slot >= 0) {
       const double t = block_sum_narrow(s, red);
       if (threadIdx.x == 0) {
         const double te = t + b.we[0];
@@ -135,8 +152,9 @@ __global__ void __launch_bounds__(512, 2) mom_pass_c_kernel(Es1dConst c, Es1dFp6
     }
     return;
   }
-  double *table = sm, *F = sm + table_words<ORDER>(nc);
-  unsigned *T = (unsigned *)(F + (nc + 1) / 2 * 2);
+  const MomShared<ORDER> m_(c, sm);
+  double *table = m_.table, *F = m_.F;
+  unsigned *T = m_.T, *W = m_.W;
   const int copies = c.copies;
   clear_fixed(T, 2 * nc * (ORDER + 1) * copies);
   griddep_wait();
@@ -144,13 +162,18 @@ __global__ void __launch_bounds__(512, 2) mom_pass_c_kernel(Es1dConst c, Es1dFp6
   const int64_t end = chunk_end(c);
   int64_t p = blockIdx.x * c.chunk + threadIdx.x;
   MarkerC<SCHEME> m(b, p, p < end);
+  unsigned *track = b.amax + (2 + par) * nc;
+  const ScaleWords words(b.amax + (2 + (par ^ 1)) * nc, track, nc);
   load_estar<SCHEME>(c, b, par, FOLD ? c.hdt_qm[0] : 1.0, F);
-  const FixedScale fs(b.amax[par], copies);
+  if (!c.late) words.store(W);
   const double scale = FOLD ? c.qw_h[0] : 1.0;
-  unsigned am = 0;
   __syncthreads();
   build_poly<ORDER>(table, F, nc);
   __syncthreads();
+  if (c.late) {
+    words.store(W);
+    __syncthreads();
+  }
   unsigned *Tl = T + (threadIdx.x & (copies - 1));
   const double hdt = c.hdt;
   for (; p < end; p += blockDim.x, m = MarkerC<SCHEME>(b, p, p < end)) {
@@ -171,13 +194,12 @@ __global__ void __launch_bounds__(512, 2) mom_pass_c_kernel(Es1dConst c, Es1dFp6
     b.sd[p] = H.d;
     double A = vs;
     if (!FOLD) A *= b.w ? c.q_h[s] * b.w[p] : c.qw_h[s];
-    am = max(am, abs_hi(A));
-    add_moments<ORDER>(Tl + (size_t)H.i * 2 * (ORDER + 1) * copies, copies, fs, H, A, scale, b.J2[par], &b.Jt[2 + par], nc);
+    add_moments<ORDER>(Tl + (size_t)H.i * 2 * (ORDER + 1) * copies, copies, W + H.i, track + H.i,
+                       c.decay & 2, H, A, scale, b.J2[par], &b.Jt[2 + par], nc);
   }
   griddep_launch_dependents();
-  flush_amax(am, &b.amax[2 + par]);
   __syncthreads();
-  flush_moments<ORDER>(T, copies, nc, scale * fs.unit(), b.J2[par], &b.Jt[2 + par]);
+  flush_moments<ORDER>(T, W, copies, nc, scale, b.J2[par], &b.Jt[2 + par]);
 }
 
 template <int ORDER, int SCHEME, bool FOLD>
@@ -194,28 +216,31 @@ __global__ void __launch_bounds__(512, 2) mom_pass_e_kernel(Es1dConst c, Es1dFp6
     const double mean = c.remove_mean ? b.Jt[2 + par] * c.inv_nc : 0.0;
     double we = 0.0;
     for (int i = threadIdx.x; i < nc; i += blockDim.x) {
+      const unsigned e = __ldcg(b.amax + (2 + par) * nc + i);
       const double en = E[i] - c.dt * (J2[i] - mean);
       b.E[par ^ 1][i] = en;
       b.J2[par ^ 1][i] = 0.0;
+      b.amax[(2 + (par ^ 1)) * nc + i] = scale_start(e, c.decay);
       we = fma(en, en, we);
     }
     const double t = block_sum_narrow(we, red);
     if (threadIdx.x == 0) {
       b.we[0] = 0.5 * c.h * t;
       b.Jt[2 + (par ^ 1)] = 0.0;
-      b.amax[2 + (par ^ 1)] = 0u;
     }
     return;
   }
-  double *table = sm, *F = sm + table_words<ORDER>(nc);
-  unsigned *T = (unsigned *)(F + (nc + 1) / 2 * 2);
+  const MomShared<ORDER> m_(c, sm);
+  double *table = m_.table, *F = m_.F;
+  unsigned *T = m_.T, *W = m_.W;
   const int copies = c.copies;
   if (SCHEME == 2) clear_fixed(T, 2 * nc * (ORDER + 1) * copies);
   griddep_wait();
   const int64_t end = chunk_end(c);
   int64_t p = blockIdx.x * c.chunk + threadIdx.x;
   MarkerE m(b, p, p < end);
-  const FixedScale fs(b.amax[2 + par], copies);
+  unsigned *track = b.amax + (par ^ 1) * nc;
+  const ScaleWords words(b.amax + par * nc, track, SCHEME == 2 ? nc : 0);
   const double scale = FOLD ? c.qw_h[0] : 1.0;
   {
     // 2 k E^{n+1/2} = 2 k E^n - k dt (j - <j>)
@@ -223,13 +248,18 @@ __global__ void __launch_bounds__(512, 2) mom_pass_e_kernel(Es1dConst c, Es1dFp6
     const double mean = c.remove_mean ? b.Jt[2 + par] * c.inv_nc : 0.0;
     for (int i = threadIdx.x; i < nc; i += blockDim.x) F[i] = fma(kj, J2[i] - mean, k2 * E[i]);
   }
+  if (!c.late) words.store(W);
   __syncthreads();
   build_poly<ORDER>(table, F, nc);
   __syncthreads();
+  if (SCHEME == 2 && c.late) {
+    words.store(W);
+    __syncthreads();
+  }
   unsigned *Tl = T + (threadIdx.x & (copies - 1));
   const double hdt = c.hdt;
   double ke = 0.0;
-  unsigned nfb = 0, am = 0;
+  unsigned nfb = 0;
   for (; p < end; p += blockDim.x, m = MarkerE(b, p, p < end)) {
     const int s = FOLD ? 0 : species_of(c, p);
     const double x = m.x, v = m.v, vs = m.vs;
@@ -271,35 +301,46 @@ __global__ void __launch_bounds__(512, 2) mom_pass_e_kernel(Es1dConst c, Es1dFp6
       b.sds[p] = N.d;
       double A = vn;
       if (!FOLD) A *= b.w ? c.q_h[s] * wp : c.qw_h[s];
-      am = max(am, abs_hi(A));
-      add_moments<ORDER>(Tl + (size_t)N.i * 2 * (ORDER + 1) * copies, copies, fs, N, A, scale, b.J1[par ^ 1], &b.Jt[par ^ 1], nc);
-    } else {
-      am = max(am, abs_hi(FOLD ? vn : (b.w ? c.q_h[s] * wp : c.qw_h[s]) * vn));
+      add_moments<ORDER>(Tl + (size_t)N.i * 2 * (ORDER + 1) * copies, copies, W + N.i, track + N.i,
+                         c.decay & 1, N, A, scale, b.J1[par ^ 1], &b.Jt[par ^ 1], nc);
     }
   }
   griddep_launch_dependents();
-  flush_amax(am, &b.amax[par ^ 1]);
   nfb = __reduce_add_sync(0xffffffffu, nfb);
   if ((threadIdx.x & 31) == 0 && nfb) atomicAdd(&b.fallback[slot], (unsigned long long)nfb);
   const double t = block_sum_narrow(ke, red);   // (its barriers order the tile before the flush)
   if (threadIdx.x == 0) b.ke_part[blockIdx.x] = FOLD ? c.half_mw[0] * t : t;
   if (SCHEME == 2)
-    flush_moments<ORDER>(T, copies, nc, scale * fs.unit(), b.J1[par ^ 1],
-                         &b.Jt[par ^ 1]);
+    flush_moments<ORDER>(T, W, copies, nc, scale, b.J1[par ^ 1], &b.Jt[par ^ 1]);
 }
 
-// The largest |amount| of the current state's deposits to *amax (zero before).
+// The point of x^n + dt/2 v^n, with the rounding that every kernel of this form uses.
+template <int ORDER>
+__device__ __forceinline__ Point64<ORDER> mom_xstar(const Es1dConst &c, double x, double v,
+                                                    unsigned *err) {
+  return Point64<ORDER>(__dmul_rn(wrap_fast(__fma_rn(c.hdt, v, x), c.L, err), c.inv_h), c.nc);
+}
+
+// The nodes' largest |amounts| of the current state's deposits to the scales (zero
+// before) of J1, parity par, and of J2 (v* is near v).
+template <int ORDER>
 __global__ void __launch_bounds__(512, 2) mom_absmax_kernel(Es1dConst c, Es1dFp64Bufs b,
-                                                            unsigned *amax) {
-  unsigned am = 0;
+                                                            int par) {
+  __shared__ unsigned W[kMomMaxNodes];
+  clear_largest(W, c.nc);
+  __syncthreads();
   const int64_t end = chunk_end(c);
   for (int64_t p = blockIdx.x * c.chunk + threadIdx.x; p < end; p += blockDim.x) {
-    double A = b.v[p];
+    const double v = b.v[p];
     const int s = species_of(c, p);
+    double A = v;
     if (!c.fold) A *= b.w ? c.q_h[s] * b.w[p] : c.qw_h[s];
-    am = max(am, abs_hi(A));
+    raise_largest(W + mom_xstar<ORDER>(c, b.x[p], v, b.err).i, abs_hi(A) >> 20);
   }
-  flush_amax(am, amax);
+  __syncthreads();
+  flush_largest(W, b.amax + par * c.nc, c.nc);
+  flush_largest(W, b.amax + 2 * c.nc, c.nc);
+  flush_largest(W, b.amax + 3 * c.nc, c.nc);
 }
 
 // j^{n,*} of the current state (ESEC2 start-up and after a state change).
@@ -308,27 +349,28 @@ __global__ void __launch_bounds__(512, 2) mom_deposit_initial_kernel(Es1dConst c
                                                                      int par) {
   extern __shared__ __align__(16) double sm[];
   const int nc = c.nc;
-  unsigned *T = (unsigned *)(sm + table_words<ORDER>(nc) + (nc + 1) / 2 * 2);
+  const MomShared<ORDER> m_(c, sm);
+  unsigned *T = m_.T, *W = m_.W;
   const int copies = c.copies;
   clear_fixed(T, 2 * nc * (ORDER + 1) * copies);
+  ScaleWords(b.amax + par * nc, nullptr, nc).store(W);
   __syncthreads();
   unsigned *Tl = T + (threadIdx.x & (copies - 1));
-  const FixedScale fs(b.amax[par], copies);
   const double scale = c.fold ? c.qw_h[0] : 1.0;
   const int64_t end = chunk_end(c);
   for (int64_t p = blockIdx.x * c.chunk + threadIdx.x; p < end; p += blockDim.x) {
     const int s = species_of(c, p);
     const double v = b.v[p];
-    const Point64<ORDER> N(
-        __dmul_rn(wrap_fast(__fma_rn(0.5 * c.dt, v, b.x[p]), c.L, b.err), c.inv_h), nc);
+    const Point64<ORDER> N = mom_xstar<ORDER>(c, b.x[p], v, b.err);
     b.sis[p] = N.i;
     b.sds[p] = N.d;
     double A = v;
     if (!c.fold) A *= b.w ? c.q_h[s] * b.w[p] : c.qw_h[s];
-    add_moments<ORDER>(Tl + (size_t)N.i * 2 * (ORDER + 1) * copies, copies, fs, N, A, scale, b.J1[par], &b.Jt[par], nc);
+    add_moments<ORDER>(Tl + (size_t)N.i * 2 * (ORDER + 1) * copies, copies, W + N.i, nullptr, 0, N,
+                       A, scale, b.J1[par], &b.Jt[par], nc);
   }
   __syncthreads();
-  flush_moments<ORDER>(T, copies, nc, scale * fs.unit(), b.J1[par], &b.Jt[par]);
+  flush_moments<ORDER>(T, W, copies, nc, scale, b.J1[par], &b.Jt[par]);
 }
 
 template <typename F>
@@ -342,10 +384,11 @@ void dispatch_mom(const Es1dConst &c, F f) {
   else c.scheme == 1 ? fold(I2(), I1()) : fold(I2(), I2());
 }
 
-size_t mom_smem(const Es1dConst &c) {
-  const size_t words = (size_t)(c.order == 1 ? 2 : 4) + (size_t)(c.order + 1) * c.copies;
-  return sizeof(double) * (words * c.nc + (c.nc + 1) / 2 * 2);
+size_t mom_smem(const Es1dConst &c, int copies, bool late) {
+  const size_t words = (size_t)(c.order == 1 ? 2 : 4) + (size_t)(c.order + 1) * copies;
+  return sizeof(double) * (words * c.nc + (c.nc + 1) / 2 * 2) + (late ? 0 : sizeof(unsigned) * c.nc);
 }
+size_t mom_smem(const Es1dConst &c) { return mom_smem(c, c.copies, c.late); }
 
 }  // namespace
 
@@ -354,8 +397,10 @@ size_t mom_smem(const Es1dConst &c) {
 bool es1d_fp64_use_moments(const Es1dConst &c) { return c.nc <= kMomMaxNodes && c.passes == 0; }
 
 LaunchShape es1d_mom_shape(const Es1dConst &c, int nsm) {
-  return fixed_shape(c.n_total, nsm, 1, c.nc / 2);
+  return fixed_shape(c.n_total, nsm, 1, c.nc / 2, mom_smem(c, 1, true) <= kTwoBlockSmem ? 2 : 1);
 }
+
+bool es1d_mom_late(const Es1dConst &c) { return mom_smem(c, 1, false) > kTwoBlockSmem; }
 
 int es1d_mom_copies(const Es1dConst &c, LaunchShape ls) {
   return fixed_copies((int64_t)c.nc * (c.order + 1), (c.n_total + ls.grid - 1) / ls.grid,
@@ -369,8 +414,7 @@ cudaError_t es1d_mom_prepare(const Es1dConst &c) {
   dispatch_mom(c, [&](auto O, auto S, auto F) {
     constexpr int ORDER = decltype(O)::value, SCHEME = decltype(S)::value;
     constexpr bool FOLD = decltype(F)::value;
-    const int most = (int)(sizeof(double) * (Poly<ORDER>::kWords + 1) * kMomMaxNodes +
-                           std::max<size_t>(kMomTileBytes, sizeof(double) * (ORDER + 1) * kMomMaxNodes));
+    const size_t most = mom_smem(c);
     for (const void *k : {(const void *)mom_pass_c_kernel<ORDER, SCHEME, FOLD>,
                           (const void *)mom_pass_e_kernel<ORDER, SCHEME, FOLD>,
                           (const void *)mom_deposit_initial_kernel<ORDER>})
@@ -383,7 +427,8 @@ cudaError_t es1d_mom_prepare(const Es1dConst &c) {
 // (b.Jt and b.amax zero before) the deposits' scale and, for ESEC2, j^{n,*}
 void es1d_mom_start(const Es1dConst &c, const Es1dFp64Bufs &b, int parity, LaunchShape ls,
                     cudaStream_t st) {
-  mom_absmax_kernel<<<ls.grid, ls.block, 0, st>>>(c, b, b.amax + parity);
+  (c.order == 1 ? mom_absmax_kernel<1> : mom_absmax_kernel<2>)
+      <<<ls.grid, ls.block, 0, st>>>(c, b, parity);
   if (c.scheme == 2)
     launch_dependent(c.order == 1 ? mom_deposit_initial_kernel<1> : mom_deposit_initial_kernel<2>,
                      ls, mom_smem(c), st, false, c, b, parity);

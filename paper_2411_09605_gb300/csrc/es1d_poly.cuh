@@ -10,7 +10,7 @@ namespace pic {
 namespace {
 
 constexpr int kMomMaxNodes = 1792;        // tables and one tile (64 bytes a node at order 2) leave
-                                          // room for two blocks on an SM
+                                          // room for two blocks on an SM up to 1760 nodes
 
 // The end of this block's run of markers.
 __device__ __forceinline__ int64_t chunk_end(const Es1dConst &c) {

@@ -79,16 +79,24 @@ __device__ __forceinline__ int64_t chunk_end(const StdConst &c) {
   return e < c.n_total ? e : c.n_total;
 }
 
-// A marker's charge at P into this lane's tile copy.
+// A marker's charge at P into this lane's tile copy; the scale words W (not FOLD) lie
+// after the tile.
 template <int ORDER, bool FOLD>
-__device__ __forceinline__ void std_deposit(unsigned *Tl, const StdConst &c, const StdBufs &b,
-                                            const FixedScale &fs, int s,
-                                            int64_t p, const Point64<ORDER> &P) {
+__device__ __forceinline__ void std_deposit(unsigned *Tl, unsigned *W, const StdConst &c,
+                                            const StdBufs &b, int s, int64_t p,
+                                            const Point64<ORDER> &P) {
   unsigned *q = Tl + (size_t)P.i * 2 * (ORDER + 1) * c.copies;
-  if (FOLD)
+  if (FOLD) {
     add_unit_moments<ORDER>(q, c.copies, P, c.qw_h[0], b.rho, b.rho + c.n, c.n);
-  else
-    add_moments<ORDER>(q, c.copies, fs, P, std_qw(c, b, s, p), 1.0, b.rho, b.rho + c.n, c.n);
+  } else {
+    const double A = std_qw(c, b, s, p);
+    add_moments<ORDER>(q, c.copies, W + P.i, b.amaxn + P.i, c.decay & 2, P, A, 1.0, b.rho, b.rho + c.n,
+                       c.n);
+  }
+}
+template <int ORDER, bool FOLD>
+__device__ __forceinline__ unsigned *std_scales(unsigned *T, const StdConst &c) {
+  return FOLD ? nullptr : T + (size_t)2 * (ORDER + 1) * c.n * c.copies;
 }
 
 template <int ORDER, bool FOLD>
@@ -96,11 +104,12 @@ __global__ void __launch_bounds__(kFixedMaxThreads, 2) std_step_kernel(StdConst 
   extern __shared__ __align__(16) double sm[];
   __shared__ double red[kRedWords];
   const int n = c.n, copies = c.copies;
-  unsigned *T = (unsigned *)(sm + (ORDER + 1) * n);
+  unsigned *T = (unsigned *)(sm + (ORDER + 1) * n), *W = std_scales<ORDER, FOLD>(T, c);
   clear_fixed(T, 2 * (ORDER + 1) * n * copies);
   griddep_wait();
+  const ScaleWords words(b.amax, b.amaxn, FOLD ? 0 : n);
   build_poly_std<ORDER>(sm, b.E, n, FOLD ? c.dt_qm[0] : 1.0);
-  const FixedScale fs(FOLD ? 0u : *b.amax, copies);
+  words.store(W);
   unsigned *Tl = T + (threadIdx.x & (copies - 1));
   __syncthreads();
   double ke = 0.0;
@@ -120,22 +129,28 @@ __global__ void __launch_bounds__(kFixedMaxThreads, 2) std_step_kernel(StdConst 
     const Point64<ORDER> P(__dmul_rn(x1, c.inv_h), n);
     b.si[p] = P.i;   // the next step gathers there
     b.sd[p] = P.d;
-    std_deposit<ORDER, FOLD>(Tl, c, b, fs, s, p, P);
+    std_deposit<ORDER, FOLD>(Tl, W, c, b, s, p, P);
   }
   griddep_launch_dependents();
   if (!isfinite(ke)) atomicOr(b.err, kErrNonfinite);
   const double kb = block_sum_narrow(ke, red);   // (its barriers order the tile's sums)
   if (threadIdx.x == 0) b.ke_part[blockIdx.x] = FOLD ? 0.5 * c.half_m[0] * c.w0[0] * kb : kb;
-  flush_moments<ORDER>(T, copies, n, FOLD ? c.qw_h[0] * kUnitTerm : fs.unit(), b.rho, b.rho + n);
+  flush_moments<ORDER, 1, !FOLD>(T, W, copies, n, FOLD ? c.qw_h[0] : 1.0, b.rho, b.rho + n);
 }
 
-// The largest |charge| of the markers (high word) to *amax (zero before).
+// The nodes' largest |charges| to amax and amaxn (zero before).
+template <int ORDER>
 __global__ void __launch_bounds__(kFixedMaxThreads, 2) std_amax_kernel(StdConst c, StdBufs b) {
-  unsigned am = 0;
+  __shared__ unsigned W[kStdMaxNodes];
+  clear_largest(W, c.n);
+  __syncthreads();
   const int64_t end = chunk_end(c);
   for (int64_t p = blockIdx.x * c.chunk + threadIdx.x; p < end; p += blockDim.x)
-    am = max(am, abs_hi(std_qw(c, b, species_of_std(c, p), p)));
-  flush_amax(am, b.amax);
+    raise_largest(W + Point64<ORDER>(__dmul_rn(b.x[p], c.inv_h), c.n).i,
+                  abs_hi(std_qw(c, b, species_of_std(c, p), p)) >> 20);
+  __syncthreads();
+  flush_largest(W, b.amax, c.n);
+  flush_largest(W, b.amaxn, c.n);
 }
 
 // The charge and the points of x^0.
@@ -143,10 +158,10 @@ template <int ORDER, bool FOLD>
 __global__ void __launch_bounds__(kFixedMaxThreads, 2) std_charge_kernel(StdConst c, StdBufs b) {
   extern __shared__ __align__(16) double sm[];
   const int n = c.n, copies = c.copies;
-  unsigned *T = (unsigned *)(sm + (ORDER + 1) * n);
+  unsigned *T = (unsigned *)(sm + (ORDER + 1) * n), *W = std_scales<ORDER, FOLD>(T, c);
   clear_fixed(T, 2 * (ORDER + 1) * n * copies);
+  ScaleWords(b.amax, b.amaxn, FOLD ? 0 : n).store(W);
   __syncthreads();
-  const FixedScale fs(FOLD ? 0u : *b.amax, copies);
   unsigned *Tl = T + (threadIdx.x & (copies - 1));
   const int64_t end = chunk_end(c);
   for (int64_t p = blockIdx.x * c.chunk + threadIdx.x; p < end; p += blockDim.x) {
@@ -154,10 +169,10 @@ __global__ void __launch_bounds__(kFixedMaxThreads, 2) std_charge_kernel(StdCons
     const Point64<ORDER> P(__dmul_rn(b.x[p], c.inv_h), n);
     b.si[p] = P.i;
     b.sd[p] = P.d;
-    std_deposit<ORDER, FOLD>(Tl, c, b, fs, s, p, P);
+    std_deposit<ORDER, FOLD>(Tl, W, c, b, s, p, P);
   }
   __syncthreads();
-  flush_moments<ORDER>(T, copies, n, FOLD ? c.qw_h[0] * kUnitTerm : fs.unit(), b.rho, b.rho + n);
+  flush_moments<ORDER, 1, !FOLD>(T, W, copies, n, FOLD ? c.qw_h[0] : 1.0, b.rho, b.rho + n);
 }
 
 // E^{n+1} into En from rho [n] and its total rho[n]: block 0 writes TE^n (slot >= 0)
@@ -175,6 +190,10 @@ __global__ void __launch_bounds__(kStdSolveThreads) std_solve_kernel(StdConst c,
   griddep_launch_dependents();
   if (blockIdx.x == 0) {
     for (int i = threadIdx.x; i <= n; i += blockDim.x) b.rhon[i] = 0.0;
+    // (the last markers' scales have been used: their place takes the next markers'
+    // largest charges)
+    for (int i = threadIdx.x; i < n && !c.fold; i += blockDim.x)
+      b.amax[i] = scale_start(b.amaxn[i], c.decay);
     if (slot < 0) return;
     double t = 0.0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) t = fma(0.5 * c.h * b.E[i], b.E[i], t);
@@ -253,7 +272,8 @@ __global__ void std_response_kernel(StdConst c, StdBufs b) {
 }
 
 size_t std_smem(const StdConst &c, int copies) {
-  return sizeof(double) * (size_t)(c.order + 1) * (1 + (size_t)copies) * c.n;
+  return sizeof(double) * (size_t)(c.order + 1) * (1 + (size_t)copies) * c.n +
+         (c.fold ? 0 : sizeof(unsigned) * c.n);
 }
 size_t std_solve_smem(const StdConst &c) { return sizeof(double) * 2 * (size_t)c.n; }
 
@@ -312,9 +332,10 @@ void std_field(const StdConst &c, const StdBufs &b, int slot, LaunchShape lp, cu
   std_solve(c, b, slot, lp, st, true);
 }
 
-// (rho, rhon and amax zero before) the charge of x^0 and E^0 into b.En.
+// (rho, rhon, amax and amaxn zero before) the charge of x^0 and E^0 into b.En.
 void std_start_field(const StdConst &c, const StdBufs &b, LaunchShape lp, cudaStream_t st) {
-  if (!c.fold) std_amax_kernel<<<lp.grid, lp.block, 0, st>>>(c, b);
+  if (!c.fold)
+    (c.order == 1 ? std_amax_kernel<1> : std_amax_kernel<2>)<<<lp.grid, lp.block, 0, st>>>(c, b);
   dispatch_std(c, [&](auto O, auto F) {
     std_charge_kernel<decltype(O)::value, decltype(F)::value>
         <<<lp.grid, lp.block, std_smem(c, c.copies), st>>>(c, b);

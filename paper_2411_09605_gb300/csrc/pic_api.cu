@@ -676,8 +676,11 @@ int init_mixed(pic_handle *h, bool solve_e0) {
   return PIC_OK;
 }
 
+// The moment passes' totals and largest amounts, in doubles.
+size_t mom_scalar_words(const Es1dConst &c) { return 4 + 2 * (size_t)c.nc; }
+
 // What the first step of an FP64 1D state needs beside its zero currents:
-// j^{n,*} (ESEC2), and the moment passes' deposit scale.
+// j^{n,*} (ESEC2), and the moment passes' deposit scales.
 void start_es1d_fp64(pic_handle *h, int par) {
   if (h->mom)
     es1d_mom_start(h->c1, h->b1, par, h->lmom, h->st);
@@ -723,6 +726,7 @@ int init_es1d(pic_handle *h, const pic_species *species, const double *E0) {
   CUDA_TRY(es1d_fp64_prepare(c));
   if (h->mom) {
     h->lmom = es1d_mom_shape(c, h->nsm);
+    c.late = es1d_mom_late(c);
     c.copies = es1d_mom_copies(c, h->lmom);
     c.chunk = es1d_mom_chunk(c, h->lmom);
     CUDA_TRY(es1d_mom_prepare(c));
@@ -754,10 +758,10 @@ int init_es1d(pic_handle *h, const pic_species *species, const double *E0) {
       ((rc = h->alloc(h->mom ? &b.sds : &b.sws, nsh)) || (rc = h->alloc(&b.sis, h->N))))
     return rc;
   if (h->mom) {
-    // Jt [4] and amax [4] in one block, cleared together
-    if ((rc = h->alloc(&b.Jt, 6))) return rc;
+    // Jt [4] and amax [4][nc] in one block, cleared together
+    if ((rc = h->alloc(&b.Jt, mom_scalar_words(c)))) return rc;
     b.amax = (unsigned *)(b.Jt + 4);
-    CUDA_TRY(cudaMemsetAsync(b.Jt, 0, sizeof(double) * 6, h->st));
+    CUDA_TRY(cudaMemsetAsync(b.Jt, 0, sizeof(double) * mom_scalar_words(c), h->st));
   }
   b.w = nullptr;
   if (h->weighted && (rc = h->alloc(&b.w, h->N))) return rc;
@@ -880,7 +884,7 @@ int restart_es1d(pic_handle *h, bool particles_changed) {
     CUDA_TRY(cudaMemsetAsync(b.J1[k], 0, sizeof(double) * h->c1.nc, h->st));
     CUDA_TRY(cudaMemsetAsync(b.J2[k], 0, sizeof(double) * h->c1.nc, h->st));
   }
-  if (h->mom) CUDA_TRY(cudaMemsetAsync(b.Jt, 0, sizeof(double) * 6, h->st));
+  if (h->mom) CUDA_TRY(cudaMemsetAsync(b.Jt, 0, sizeof(double) * mom_scalar_words(h->c1), h->st));
   start_es1d_fp64(h, par);
   CUDA_TRY(cudaGetLastError());
   validate_1d_kernel<<<h->ls.grid, 256, 0, h->st>>>(b.x, b.v, h->N, h->c1.L, b.err);
@@ -1146,10 +1150,12 @@ int restart_std(pic_handle *h) {
   CUDA_TRY(cudaGetLastError());
   CUDA_TRY(cudaMemsetAsync(b.rho, 0, sizeof(double) * (h->cs.n + 1), h->st));
   CUDA_TRY(cudaMemsetAsync(b.rhon, 0, sizeof(double) * (h->cs.n + 1), h->st));
-  CUDA_TRY(cudaMemsetAsync(b.amax, 0, sizeof(unsigned), h->st));
+  CUDA_TRY(cudaMemsetAsync(b.amax, 0, sizeof(unsigned) * h->cs.n, h->st));
+  CUDA_TRY(cudaMemsetAsync(b.amaxn, 0, sizeof(unsigned) * h->cs.n, h->st));
   std_start_field(h->cs, b, h->lsd, h->st);
   std::swap(b.E, b.En);
   std::swap(b.rho, b.rhon);
+  std::swap(b.amax, b.amaxn);
   std_kick_back(h->cs, b, h->lsd, h->st);
   CUDA_TRY(cudaGetLastError());
   h->launches += 4 + !h->cs.fold;
@@ -1196,7 +1202,8 @@ int init_std(pic_handle *h, const pic_species *species) {
   if ((rc = h->alloc(&b.sd, h->N)) || (rc = h->alloc(&b.si, h->N)) || (rc = h->alloc(&b.E, n)) ||
       (rc = h->alloc(&b.En, n)) || (rc = h->alloc(&b.rho, n + 1)) ||
       (rc = h->alloc(&b.rhon, n + 1)) || (rc = h->alloc(&b.resp, n)) ||
-      (rc = h->alloc(&b.amax, 1)) || (rc = h->alloc(&b.ke_part, (size_t)h->lsd.grid)) ||
+      (rc = h->alloc(&b.amax, n)) || (rc = h->alloc(&b.amaxn, n)) ||
+      (rc = h->alloc(&b.ke_part, (size_t)h->lsd.grid)) ||
       (rc = h->alloc(&b.fallback, kStepsCap)) || (rc = h->alloc(&b.te, kStepsCap)) ||
       (rc = h->alloc(&b.err, 1)) || (rc = h->alloc(&h->ids, h->N)) ||
       (rc = h->alloc(&h->std_part, (size_t)h->lsd.grid * h->nsp + 1)))
@@ -1253,7 +1260,7 @@ int restart_em1d(pic_handle *h, bool markers_changed = true) {
     em1m_start(h->c1e, b, h->c1m, mb, h->le, h->st);
     h->launches += 1 + (markers_changed ? 2 : 1) + 2 * (h->c1e.scheme == 2);
   } else {
-    CUDA_TRY(cudaMemsetAsync(b.amax, 0, sizeof(unsigned) * 2, h->st));
+    CUDA_TRY(cudaMemsetAsync(b.amax, 0, sizeof(unsigned) * 8 * h->c1e.n, h->st));
     em1d_start(h->c1e, b, h->le, h->st);
     h->launches += 3 + (h->c1e.scheme == 2);
   }
@@ -1404,7 +1411,7 @@ int init_em1d(pic_handle *h, const pic_species *species, const double *E0, const
   b.si = b.sis = nullptr;
   b.amax = nullptr;
   if (!h->mixed && ((rc = h->alloc(&b.sd, h->N)) || (rc = h->alloc(&b.si, h->N)) ||
-                    (rc = h->alloc(&b.amax, 2))))
+                    (rc = h->alloc(&b.amax, 8 * n))))
     return rc;
   if (!h->mixed && cfg.scheme == 2 &&
       ((rc = h->alloc(&b.sds, h->N)) || (rc = h->alloc(&b.sis, h->N))))
@@ -1677,10 +1684,12 @@ int pic_step_async(pic_handle *h, int nsteps) {
   }
   for (int k = 0; k < nsteps && h->stdp; k++) {
     const int slot = h->pending;
+    h->cs.decay = scale_decay(h->steps_done);
     CUDA_TRY(h->timed_launch(1, [&] { std_markers(h->cs, h->bs, h->lsd, h->st); }));
     CUDA_TRY(h->timed_launch(4, [&] { std_field(h->cs, h->bs, slot, h->lsd, h->st); }));
     std::swap(h->bs.E, h->bs.En);
     std::swap(h->bs.rho, h->bs.rhon);
+    std::swap(h->bs.amax, h->bs.amaxn);
     h->launches += 2;
     h->steps_done++;
     h->pending++;
@@ -1694,6 +1703,7 @@ int pic_step_async(pic_handle *h, int nsteps) {
         em1m_pass_e(h->c1e, e, h->c1m, h->b1m, slot, h->le, h->st);
       }));
     } else {
+      h->c1e.decay = scale_decay(h->steps_done);
       CUDA_TRY(h->timed_launch(0, [&] { em1d_pass_c(h->c1e, e, h->le, h->st); }));
       CUDA_TRY(h->timed_launch(1, [&] { em1d_pass_e(h->c1e, e, slot, h->le, h->st); }));
     }
@@ -1817,6 +1827,7 @@ int pic_step_async(pic_handle *h, int nsteps) {
       }));
       if (h->cm.mode == 2) swap_sorted_output(h);
     } else {
+      h->c1.decay = scale_decay(h->steps_done);
       CUDA_TRY(h->timed_launch(0, [&] {
         if (h->mom)
           es1d_mom_pass_c(h->c1, b, h->steps_done, h->pending, h->lmom, h->st);
@@ -2338,7 +2349,7 @@ int grad_rerun_mom(pic_handle *h, int seg, int s0, int s1, bool all, double *sca
     b.sds = sds;
     b.sis = sis;
   }
-  CUDA_TRY(cudaMemsetAsync(scal, 0, sizeof(double) * 6, h->st));
+  CUDA_TRY(cudaMemsetAsync(scal, 0, sizeof(double) * mom_scalar_words(h->c1), h->st));
   CUDA_TRY(cudaMemsetAsync(J2, 0, sizeof(double) * 2 * nc, h->st));
   CUDA_TRY(cudaMemsetAsync(grad_rec_j1(h, 0), 0, sizeof(double) * nc, h->st));
   auto state = [&](int j) {
@@ -2366,14 +2377,14 @@ int grad_backward_mom(pic_handle *h, const double *Ebar, const double *xbar, con
   const size_t N = (size_t)h->N, nc = (size_t)h->c1.nc, rec = grad_rec_words(h);
   const int seglen = std::min(g.every, g.nsteps);
   const size_t words = es1d_rev_table_words(h->c1);
-  constexpr size_t kScal = 16;
+  const size_t kScal = 5 + mom_scalar_words(h->c1) + 3 * nc;
   if (!g.grid) CUDA_TRY(cudaMalloc(&g.grid, sizeof(double) * (7 * nc + kScal)));
   if (!g.mk) CUDA_TRY(cudaMalloc(&g.mk, sizeof(double) * 9 * N + 16));
   CUDA_TRY(grad_room(&g.seg, &g.seg_cap, (seglen + 1) * rec));
   CUDA_TRY(grad_room(&g.tab, &g.tab_cap, seglen * words));
   CUDA_TRY(es1d_rev_prepare(h->c1));
   CUDA_TRY(cudaMemsetAsync(g.grid, 0, sizeof(double) * (7 * nc + kScal), h->st));
-  // scalars: 6 of the re-run's passes, 5 sums and 8 words of the reverse
+  // scalars: the re-run's passes', five sums and the nodes' six words of the reverse
   double *scal = g.grid + 7 * nc, *mk = g.mk;
   Es1dRevBufs r{};
   r.w = h->b1.w;
@@ -2384,9 +2395,9 @@ int grad_backward_mom(pic_handle *h, const double *Ebar, const double *xbar, con
     r.Es[k] = g.grid + (3 + k) * nc;
   }
   double *J2 = g.grid + 5 * nc;
-  r.gtot = scal + 6;
-  r.tot = scal + 7;
-  r.mx = (unsigned *)(scal + 11);
+  r.gtot = scal + mom_scalar_words(h->c1);
+  r.tot = r.gtot + 1;
+  r.mx = (unsigned *)(r.gtot + 5);
   r.xb = mk;
   r.vb = mk + N;
   r.wb = mk + 2 * N;
@@ -2414,6 +2425,7 @@ int grad_backward_mom(pic_handle *h, const double *Ebar, const double *xbar, con
   CUDA_TRY(input(vbar, r.vb, N, &r.vin));
   int par = 0;
   if (r.vin) {
+    r.x = h->b1.x;
     es1d_rev_start(h->c1, r, par, h->lmom, h->st);
     CUDA_TRY(cudaGetLastError());
     h->launches += 1;
@@ -2439,6 +2451,7 @@ int grad_backward_mom(pic_handle *h, const double *Ebar, const double *xbar, con
       r.v = state(k).v;
       r.v1 = state(k + 1).v;
       r.tables = g.tab + (k - s0) * words;
+      r.decay = scale_decay(k);
       es1d_rev_step(h->c1, r, par, k + 1 == g.nsteps, k + 1 == s1, h->lmom, h->st);
     }
     CUDA_TRY(cudaGetLastError());

@@ -60,6 +60,8 @@ struct Es1dConst {
   // single uniformly weighted species are applied once per sum (fold)
   int fold;
   int copies;                    // tile copies of a block (a power of two)
+  int late;                      // the nodes' scale words take the place of the field
+  int decay;                     // whether the nodes' scales fall (scale_decay)
   int64_t chunk;                 // markers of a block
   double inv_nc;                 // 1 / nc
   double hdt;                    // dt/2 (a constant: formed in a kernel it is formed per marker)
@@ -233,6 +235,7 @@ struct Em1dConst {
   int gamma_on;
   int nsp;
   int copies;       // FP64 passes: copies of the shared current tile (power of two, <= 32)
+  int decay;        // FP64 passes: whether the nodes' scales fall (scale_decay)
   int fold;         // one uniformly weighted species: its factors go to tables and sums
   int64_t chunk;    // FP64 passes: markers of a block
   int direct;       // 1: the direct field solve (n <= kEm1DirectNodes), a service block first
@@ -254,7 +257,8 @@ struct Em1dBufs {
   int *si;                   // [N] the node (pass C -> pass E)
   double *sds;               // ESEC2: the next step's y* (pass E or the initial deposit
   int *sis;                  // -> pass C), as sd / si; null: formed again
-  unsigned *amax;            // [2] largest amounts deposited into J1 and J2 (high words)
+  unsigned *amax;            // [2][2][n][2] exponents of the nodes' largest amounts in J1 and J2:
+                             // of the last pass and of the present one
   double *E, *En;            // E^n, E^{n+1}: [2][n] (Ex, Ey); swapped after each step
   double *B, *Bn;            // Bz^n, Bz^{n+1}: [n]
   double *Es, *Bs;           // E*, B* of the half step
@@ -280,6 +284,7 @@ struct StdConst {
   int order;
   int nsp;
   int copies;       // copies of the shared charge tile (power of two, <= 32)
+  int decay;        // whether the nodes' scales fall (scale_decay)
   int fold;         // one uniformly weighted species: its factors go to tables and sums
   int64_t chunk;    // markers of a block
   int passes;       // 1-2-1 filter passes on the charge
@@ -302,7 +307,8 @@ struct StdBufs {
   double *rho, *rhon;    // [n + 1] charge of the next positions and its total; the other
                          // buffer is cleared meanwhile, swapped after each step
   double *resp;          // [n] E of a unit charge at node 0
-  unsigned *amax;        // [1] the largest |charge| (high word; several species, weights)
+  unsigned *amax, *amaxn;   // [n] exponents of the nodes' largest charges (several species,
+                            // weights) of the last markers and the next; swapped as rho
   double *ke_part;       // [particle blocks]
   unsigned long long *fallback;
   double *te;
@@ -400,7 +406,7 @@ struct Es1dFp64Bufs {
   double *sd, *sds;         // moment passes: [N] the offset from node si (sis) in
                             // place of the weights sw (sws); null otherwise
   double *Jt;               // moment passes: totals of J1[0], J1[1], J2[0], J2[1]
-  unsigned *amax;           // and the largest amounts deposited into them (high words)
+  unsigned *amax;           // and [4][nc] the exponents of the nodes' largest amounts in them
   double *E[2];             // ping-pong E^n / E^{n+1}
   double *J1[2];            // j^{n,*} (ESEC2), indexed by step parity
   double *J2[2];            // j^{*,n+1/2}
@@ -450,6 +456,13 @@ cudaError_t allow_shared(K *kern, size_t bytes) {
                               room);
 }
 
+// Whether a step (bit 0) and the one before it (bit 1) let the scales of the fixed-point
+// deposits fall by one exponent (fixed_moments.cuh).
+constexpr int kScaleSteps = 8;
+inline int scale_decay(int64_t step) {
+  return (step % kScaleSteps == 0) | (step % kScaleSteps == 1) << 1;
+}
+
 // Sets the message returned by pic_last_error (pic_api.cu).
 void set_last_error(const std::string &msg);
 
@@ -477,12 +490,13 @@ struct Es1dRevBufs {
   double *G, *gtot;         // [nc] adjoint of the field and its sum
   double *Hb[2], *Es[2];    // [nc] adjoints of E^{n+1/2} and E* by step parity
   double *tot;              // [2][2] their totals
-  unsigned *mx;             // [2][4] largest amounts (high words)
+  unsigned *mx;             // [2][3][nc] exponents of the nodes' largest amounts
   double *xb, *vb, *wb;     // [N] adjoints of the markers (x in cells)
   double *ub, *yb, *u, *ap, *dy;   // [N] marker scratch
   long long *D;
   int *ix, *iy;
   int copies;               // tile copies of a block
+  int decay;                // whether the nodes' words fall (scale_decay)
   unsigned *err;
 };
 int es1d_rev_copies(const Es1dConst &c, LaunchShape ls);
@@ -503,6 +517,7 @@ cudaError_t es1d_fp64_prepare(const Es1dConst &c);
 // (ls.grid marker blocks and one service block), and their kernels' set-up.
 bool es1d_fp64_use_moments(const Es1dConst &c);
 LaunchShape es1d_mom_shape(const Es1dConst &c, int nsm);
+bool es1d_mom_late(const Es1dConst &c);
 int es1d_mom_copies(const Es1dConst &c, LaunchShape ls);
 int64_t es1d_mom_chunk(const Es1dConst &c, LaunchShape ls);
 cudaError_t es1d_mom_prepare(const Es1dConst &c);
