@@ -2323,10 +2323,22 @@ int grad_forward_mom(pic_handle *h) {
                                                      : w.own.J1[(g.start + k) & 1];
   };
   for (int k = 0; k < g.nsteps; k++) {
-    int rc;
-    if (h->pending == kStepsCap && (rc = pic_read_stats(h, 0, nullptr, nullptr, nullptr)))
-      return rc;
-    if ((rc = w.step(state(k), state(k + 1), j1(k), j1(k + 1)))) return rc;
+    int rc = PIC_OK;
+    if (h->pending == kStepsCap) rc = pic_read_stats(h, 0, nullptr, nullptr, nullptr);
+    if (!rc) rc = w.step(state(k), state(k + 1), j1(k), j1(k + 1));
+    if (!rc) continue;
+    // the handle goes on from the last state that was reached, which may lie in a record
+    // (x* of it is where the steps leave it, in the handle's own arrays)
+    const int at = (int)(h->steps_done - g.start), par = (int)(h->steps_done & 1);
+    const GradState z = state(at);
+    const double *from[4] = {z.x, z.v, z.E, j1(at)};
+    double *to[4] = {w.own.x, w.own.v, w.own.E[par], w.own.J1[par]};
+    for (int i = 0; i < 4; i++)
+      if (from[i] != to[i])
+        cudaMemcpyAsync(to[i], from[i], sizeof(double) * (i < 2 ? (size_t)h->N : nc),
+                        cudaMemcpyDeviceToDevice, h->st);
+    g.start = -1;
+    return rc;
   }
   g.held = keep && kept > 0;
   return PIC_OK;
