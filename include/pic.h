@@ -346,7 +346,9 @@ int pic_es1d_step_noalloc(const pic_config *cfg, double q, double m, double w0, 
  * pic_grad_forward steps h forward nsteps steps (as pic_step_async; pending
  * stats must have been read) and keeps the markers and field every
  * checkpoint_every steps on the device ((nsteps / checkpoint_every + 1) x
- * (2 N + nodes) doubles).
+ * (2 N + nodes) doubles) and, on grids of up to 1792 nodes, where there is room,
+ * every state of the last segment ((min(checkpoint_every, nsteps) + 1) x
+ * (2 N + 2 nodes) doubles).  After an error h is at the last step that was reached.
  *
  * pic_grad_backward takes the adjoints of the state after those steps -
  * Ebar [nodes], xbar [N], vbar [N] (host or device, NULL = zero) - and writes
@@ -354,9 +356,11 @@ int pic_es1d_step_noalloc(const pic_config *cfg, double q, double m, double w0, 
  * [N] (the derivative by each marker's weight; for a uniformly weighted
  * species the derivative by its w0 is the sum over its markers), host or
  * device, each may be NULL.  Each segment of checkpoint_every steps is
- * re-run from its checkpoint and reversed; h is left at the state after the
- * forward steps.  The step sequence must not change in between, else
- * PIC_ERR_ARG.
+ * re-run from its checkpoint (the last one only where its states were not kept)
+ * and reversed; h is left at the state after the forward steps, whose unread stats
+ * are discarded.  An error that they hold is reported, and after any error the
+ * output arrays are as they were.  The step sequence must not change in between,
+ * else PIC_ERR_ARG.
  */
 int pic_grad_forward(pic_handle *h, int nsteps, int checkpoint_every);
 int pic_grad_backward(pic_handle *h, const double *Ebar, const double *xbar, const double *vbar,

@@ -2478,12 +2478,18 @@ int grad_backward_mom(pic_handle *h, const double *Ebar, const double *xbar, con
   es1d_rev_last(h->c1, r, par ^ 1, dst[0], dst[1], dst[2], dst[3], h->lmom, h->st);
   CUDA_TRY(cudaGetLastError());
   h->launches += 1;
+  // after an error the caller's arrays stay as they are (es1d_rev_last looks itself)
+  const int rc = check_flags(h, "pic_grad_backward");
+  if (rc) return rc;
+  bool copied = false;
   for (int k = 0; k < 4; k++)
-    if (out[k] && dst[k] == own[k])
+    if (out[k] && dst[k] == own[k]) {
       CUDA_TRY(cudaMemcpyAsync(out[k], own[k], sizeof(double) * (k ? N : nc), cudaMemcpyDefault,
                                h->st));
-  CUDA_TRY(cudaStreamSynchronize(h->st));
-  return check_flags(h, "pic_grad_backward");
+      copied = true;
+    }
+  if (copied) CUDA_TRY(cudaStreamSynchronize(h->st));
+  return PIC_OK;
 }
 
 }  // namespace
@@ -2532,7 +2538,13 @@ int pic_grad_backward(pic_handle *h, const double *Ebar, const double *xbar, con
   if (g.start < 0 || h->steps_done != g.start + g.nsteps)
     return fail(PIC_ERR_ARG, "pic_grad_backward: no pic_grad_forward ends at the current step");
   if (h->mom) {
-    h->pending = 0;   // stats not read yet are discarded; the flags are checked at the end
+    // stats not read yet are discarded, but not the check of the last step's energy
+    if (h->pending) {
+      es1d_fp64_finalize(h->c1, h->b1, h->pending - 1, h->lmom.grid, h->st);
+      CUDA_TRY(cudaGetLastError());
+      h->launches += 1;
+    }
+    h->pending = 0;
     return grad_backward_mom(h, Ebar, xbar, vbar, Ebar0, xbar0, vbar0, wbar0);
   }
   int rc = pic_read_stats(h, 0, nullptr, nullptr, nullptr);

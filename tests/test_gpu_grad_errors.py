@@ -47,3 +47,25 @@ def test_forward_error_leaves_a_consistent_state(every, scheme):
     finally:
         for s in sims:
             s.close()
+
+
+@pytest.mark.parametrize("device", [False, True])
+def test_backward_reports_the_last_step(device):
+    """An energy that overflows in the last forward step, whose stats were not read: the
+    reverse reports it and leaves the outputs as they are."""
+    import torch
+    from paper_2411_09605_gb300 import pic
+    prob = W.landau(n=50, nc=8, dt=1e-6, seed=4)
+    prob.species[0].w0 = 1e300
+    sim = pic.Simulation(prob, scheme=1, E0=np.zeros(8))
+    out = [torch.full((k,), 7.0, dtype=torch.float64, device="cuda" if device else "cpu")
+           for k in (8, 50, 50, 50)]
+    try:
+        pic.pic_grad_forward(sim.h, 1, 1)
+        torch.cuda.synchronize()
+        with pytest.raises(pic.PicError) as e:
+            pic.pic_grad_backward(sim.h, None, None, np.ones(50), *out)
+        assert pic.ERRORS[e.value.code] == "PIC_ERR_NONFINITE"
+        assert all(bool((t == 7.0).all()) for t in out)
+    finally:
+        sim.close()
