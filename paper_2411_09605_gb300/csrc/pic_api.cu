@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "debug_bounds.cuh"
+#include "kernel_address.h"
 #include "pic_internal.cuh"
 
 using namespace pic;
@@ -246,21 +247,17 @@ cudaError_t ensure_copy_stream(pic_handle *h) {
   return e;
 }
 
-// p as the device addresses it: device or managed memory, or host memory that
-// is pinned and mapped into the device's address space (kernels then read or
-// write it over the host link directly, at the link's rate); null for other
-// host memory (pageable), which goes through cudaMemcpy.
+// p as the current device addresses it (kernel_address), or null: then it goes through
+// cudaMemcpy.
 template <typename T>
 T *device_view(T *p) {
   cudaPointerAttributes a;
-  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+  int device = 0;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&device) != cudaSuccess) {
     cudaGetLastError();  // an unknown pointer is not an error here
     return nullptr;
   }
-  if (a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged ||
-      a.type == cudaMemoryTypeHost)
-    return static_cast<T *>(a.devicePointer);
-  return nullptr;
+  return static_cast<T *>(kernel_address(a, device));
 }
 
 // pic_set_particles of the mixed 1D form.  Markers the device can address
