@@ -2772,7 +2772,8 @@ struct pic_batch {
   int scheme = 2;
   size_t smem = 0;
   int nitems = 0;
-  int trips = 8;  // the autotuner's target of 4-marker trips per block of a run
+  int trips = 0;  // the work list's target of 4-marker trips per block, 0: pic_batch_init's
+  int init_trips = 8;  // the one of 4, 8 and 16 nearest to that list's trips
   int threads = 1024;  // block size of the passes (256 for batches of small runs)
   bool prev_closed = false;  // the last pending step's TE was reduced already
   Es1dMixConst *d_c = nullptr;
@@ -2949,6 +2950,12 @@ int pic_batch_init(const pic_config *cfgs, const pic_species *species, int nruns
     }
   }
   b->nitems = (int)items.size();
+  {
+    double groups = 0.0;
+    for (const pic_handle *h : b->runs) groups += (double)((h->N + 3) / 4);
+    const double t = groups / b->threads / b->nitems;
+    b->init_trips = t < 5.66 ? 4 : t < 11.3 ? 8 : 16;
+  }
   if (!cfgs[0].cuda_stream) {
     // the legacy default stream cannot be captured into a graph: the batch and
     // its runs move to a stream of their own
@@ -2986,16 +2993,23 @@ int pic_batch_init(const pic_config *cfgs, const pic_species *species, int nruns
   return PIC_OK;
 }
 
-// Replaces the work list for a new trip target, within 1.4 of it (the graphs captured with the
-// old list are dropped).
-static int batch_retarget(pic_batch *b, int trips) {
+// Replaces the work list for a trip target (within 1.4 of it) or, for 0, by the one that
+// pic_batch_init makes (the graphs captured with the old list are dropped).  taken:
+// whether the list is that one now; a target that would break the tiles' bound leaves
+// the list as it is.
+static int batch_retarget(pic_batch *b, int trips, bool *taken) {
+  *taken = true;
+  if (b->trips == trips) return PIC_OK;
   std::vector<BatchItem> items;
-  std::vector<int> nbs =
-      batch_items(b->runs, trips / 1.4, std::min<double>(kBatchMostTrips, trips * 1.4), b->threads,
-                  items);
+  std::vector<int> nbs = batch_items(
+      b->runs, trips ? trips / 1.4 : 1.0,
+      trips ? std::min<double>(kBatchMostTrips, trips * 1.4) : kBatchMostTrips, b->threads, items);
   for (int r = 0; r < (int)b->runs.size(); r++) {
     const int64_t ngroups = (b->runs[r]->N + 3) / 4;
-    if (batch_trips(ngroups, nbs[r], b->threads) > kBatchMostTrips) return PIC_OK;
+    if (batch_trips(ngroups, nbs[r], b->threads) > kBatchMostTrips) {
+      *taken = false;
+      return PIC_OK;
+    }
   }
   CUDA_TRY(cudaStreamSynchronize(b->st));
   if (b->pending && !b->prev_closed) {
@@ -3040,6 +3054,7 @@ int pic_batch_autotune(pic_batch *b, int steps_per_trial, int *trips) {
   const auto key = std::make_tuple((int)b->runs.size(), lg, ncmax);
   auto it = g_batch_tuned.find(key);
   int best = b->trips;
+  bool taken = false;
   if (it != g_batch_tuned.end()) {
     best = it->second;
   } else {
@@ -3047,11 +3062,12 @@ int pic_batch_autotune(pic_batch *b, int steps_per_trial, int *trips) {
     CUDA_TRY(cudaEventCreate(&e0));
     CUDA_TRY(cudaEventCreate(&e1));
     float best_ms = 1e30f;
-    for (int t : {4, 8, 16}) {
+    for (int target : {4, 8, 16}) {
       if (b->pending + steps_per_trial > kStepsCap) break;
-      int rc = batch_retarget(b, t);
+      const int t = target == b->init_trips ? 0 : target;
+      int rc = batch_retarget(b, t, &taken);
       if (rc) return rc;
-      if (b->trips != t) continue;  // this target would break the tiles' bound
+      if (!taken) continue;
       CUDA_TRY(cudaEventRecord(e0, b->st));
       b->enqueue(steps_per_trial, b->pending);
       CUDA_TRY(cudaEventRecord(e1, b->st));
@@ -3069,11 +3085,11 @@ int pic_batch_autotune(pic_batch *b, int steps_per_trial, int *trips) {
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    g_batch_tuned[key] = best;
+    if (best_ms < 1e30f) g_batch_tuned[key] = best;
   }
-  int rc = batch_retarget(b, best);
+  int rc = batch_retarget(b, best, &taken);
   if (rc) return rc;
-  if (trips) *trips = b->trips;
+  if (trips) *trips = b->trips ? b->trips : b->init_trips;
   return PIC_OK;
 }
 
