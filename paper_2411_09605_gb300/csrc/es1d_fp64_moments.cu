@@ -132,16 +132,14 @@ __global__ void __launch_bounds__(512, 2) mom_pass_c_kernel(Es1dConst c, Es1dFp6
       clear_doubles(b.J1[par ^ 1], nc);
       if (threadIdx.x == 0) b.Jt[par ^ 1] = 0.0;
     }
-    // where the next j^{n,*}'s largest amounts start (b.amax: [4][nc], J1 and J2 by parity)
-    const unsigned *e = b.amax + par * nc;
-    unsigned *next = b.amax + (par ^ 1) * nc;
-    const unsigned e0 = (int)threadIdx.x < nc ? __ldcg(e + threadIdx.x) : 0u;
+    if (threadIdx.x == 0) b.vmax[par ^ 1] = 0u;
+    // pass E's scales, from what the pass E before recorded (all loads first)
+    const ScaleMaker<> scales(b.words, b.rec, SCHEME == 2 ? nc : 0);
+    const unsigned vmax = __ldcg(b.vmax + par);
     double s = 0.0;
     if (prev_slot >= 0)
       for (int i = threadIdx.x; i < nblk; i += blockDim.x) s += b.ke_part[i];
-    if ((int)threadIdx.x < nc) next[threadIdx.x] = scale_start(e0, c.decay);
-    for (int i = threadIdx.x + blockDim.x; i < nc; i += blockDim.x)
-      next[i] = scale_start(__ldcg(e + i), c.decay);
+    if (SCHEME == 2) scales.make((unsigned *)sm, node_reach(vmax, c.reach), c.decay);
     if (prev_slot >= 0) {
       const double t = block_sum_narrow(s, red);
       if (threadIdx.x == 0) {
@@ -162,8 +160,7 @@ __global__ void __launch_bounds__(512, 2) mom_pass_c_kernel(Es1dConst c, Es1dFp6
   const int64_t end = chunk_end(c);
   int64_t p = blockIdx.x * c.chunk + threadIdx.x;
   MarkerC<SCHEME> m(b, p, p < end);
-  unsigned *track = b.amax + (2 + par) * nc;
-  const ScaleWords words(b.amax + (2 + (par ^ 1)) * nc, track, nc);
+  const ScaleWords words(b.words + nc + 1, nc + 1);
   load_estar<SCHEME>(c, b, par, FOLD ? c.hdt_qm[0] : 1.0, F);
   if (!c.late) words.store(W);
   const double scale = FOLD ? c.qw_h[0] : 1.0;
@@ -194,12 +191,13 @@ __global__ void __launch_bounds__(512, 2) mom_pass_c_kernel(Es1dConst c, Es1dFp6
     b.sd[p] = H.d;
     double A = vs;
     if (!FOLD) A *= b.w ? c.q_h[s] * b.w[p] : c.qw_h[s];
-    add_moments<ORDER>(Tl + (size_t)H.i * 2 * (ORDER + 1) * copies, copies, W + H.i, track + H.i,
-                       c.decay & 2, H, A, scale, b.J2[par], &b.Jt[2 + par], nc);
+    add_moments<ORDER>(Tl + (size_t)H.i * 2 * (ORDER + 1) * copies, copies, W + H.i, H, A, scale,
+                       b.J2[par], &b.Jt[2 + par], nc);
   }
   griddep_launch_dependents();
   __syncthreads();
-  flush_moments<ORDER>(T, W, copies, nc, scale, b.J2[par], &b.Jt[2 + par]);
+  flush_new(W, b.rec + nc, nc);
+  flush_moments<ORDER>(T, W, copies, nc, scale, b.J2[par], &b.Jt[2 + par], ScaleRange(W[nc]));
 }
 
 template <int ORDER, int SCHEME, bool FOLD>
@@ -213,14 +211,14 @@ __global__ void __launch_bounds__(512, 2) mom_pass_e_kernel(Es1dConst c, Es1dFp6
   if ((int)blockIdx.x == nblk) {   // service block: E^{n+1}, W_E, the cleared J2
     griddep_wait();
     griddep_launch_dependents();
+    const ScaleMaker<> scales(b.words + nc + 1, b.rec + nc, nc);
+    const unsigned vmax = __ldcg(b.vmax + par);
     const double mean = c.remove_mean ? b.Jt[2 + par] * c.inv_nc : 0.0;
     double we = 0.0;
     for (int i = threadIdx.x; i < nc; i += blockDim.x) {
-      const unsigned e = __ldcg(b.amax + (2 + par) * nc + i);
       const double en = E[i] - c.dt * (J2[i] - mean);
       b.E[par ^ 1][i] = en;
       b.J2[par ^ 1][i] = 0.0;
-      b.amax[(2 + (par ^ 1)) * nc + i] = scale_start(e, c.decay);
       we = fma(en, en, we);
     }
     const double t = block_sum_narrow(we, red);
@@ -228,6 +226,8 @@ __global__ void __launch_bounds__(512, 2) mom_pass_e_kernel(Es1dConst c, Es1dFp6
       b.we[0] = 0.5 * c.h * t;
       b.Jt[2 + (par ^ 1)] = 0.0;
     }
+    // the next pass C's scales, from what the last one recorded
+    scales.make((unsigned *)sm, node_reach(vmax, c.reach), c.decay);
     return;
   }
   const MomShared<ORDER> m_(c, sm);
@@ -239,8 +239,7 @@ __global__ void __launch_bounds__(512, 2) mom_pass_e_kernel(Es1dConst c, Es1dFp6
   const int64_t end = chunk_end(c);
   int64_t p = blockIdx.x * c.chunk + threadIdx.x;
   MarkerE m(b, p, p < end);
-  unsigned *track = b.amax + (par ^ 1) * nc;
-  const ScaleWords words(b.amax + par * nc, track, SCHEME == 2 ? nc : 0);
+  const ScaleWords words(b.words, SCHEME == 2 ? nc + 1 : 0);
   const double scale = FOLD ? c.qw_h[0] : 1.0;
   {
     // 2 k E^{n+1/2} = 2 k E^n - k dt (j - <j>)
@@ -259,7 +258,7 @@ __global__ void __launch_bounds__(512, 2) mom_pass_e_kernel(Es1dConst c, Es1dFp6
   unsigned *Tl = T + (threadIdx.x & (copies - 1));
   const double hdt = c.hdt;
   double ke = 0.0;
-  unsigned nfb = 0;
+  unsigned nfb = 0, vm = 0;
   for (; p < end; p += blockDim.x, m = MarkerE(b, p, p < end)) {
     const int s = FOLD ? 0 : species_of(c, p);
     const double x = m.x, v = m.v, vs = m.vs;
@@ -292,6 +291,7 @@ __global__ void __launch_bounds__(512, 2) mom_pass_e_kernel(Es1dConst c, Es1dFp6
     const double xn = wrap_fast(__fma_rn(c.dt, vs, x), c.L, b.err);
     b.xo[p] = xn;
     b.vo[p] = vn;
+    vm = max(vm, abs_hi(vn));
     const double wp = !FOLD && b.w ? b.w[p] : 1.0;
     ke = FOLD ? __fma_rn(vn, vn, ke)
                 : __fma_rn((b.w ? c.half_m[s] * wp : c.half_mw[s]) * vn, vn, ke);
@@ -301,17 +301,21 @@ __global__ void __launch_bounds__(512, 2) mom_pass_e_kernel(Es1dConst c, Es1dFp6
       b.sds[p] = N.d;
       double A = vn;
       if (!FOLD) A *= b.w ? c.q_h[s] * wp : c.qw_h[s];
-      add_moments<ORDER>(Tl + (size_t)N.i * 2 * (ORDER + 1) * copies, copies, W + N.i, track + N.i,
-                         c.decay & 1, N, A, scale, b.J1[par ^ 1], &b.Jt[par ^ 1], nc);
+      add_moments<ORDER>(Tl + (size_t)N.i * 2 * (ORDER + 1) * copies, copies, W + N.i, N, A, scale,
+                         b.J1[par ^ 1], &b.Jt[par ^ 1], nc);
     }
   }
   griddep_launch_dependents();
+  flush_vmax(vm, &b.vmax[par ^ 1]);
   nfb = __reduce_add_sync(0xffffffffu, nfb);
   if ((threadIdx.x & 31) == 0 && nfb) atomicAdd(&b.fallback[slot], (unsigned long long)nfb);
   const double t = block_sum_narrow(ke, red);   // (its barriers order the tile before the flush)
   if (threadIdx.x == 0) b.ke_part[blockIdx.x] = FOLD ? c.half_mw[0] * t : t;
-  if (SCHEME == 2)
-    flush_moments<ORDER>(T, W, copies, nc, scale, b.J1[par ^ 1], &b.Jt[par ^ 1]);
+  if (SCHEME == 2) {
+    flush_new(W, b.rec, nc);
+    flush_moments<ORDER>(T, W, copies, nc, scale, b.J1[par ^ 1], &b.Jt[par ^ 1],
+                         ScaleRange(W[nc]));
+  }
 }
 
 // The point of x^n + dt/2 v^n, with the rounding that every kernel of this form uses.
@@ -321,26 +325,37 @@ __device__ __forceinline__ Point64<ORDER> mom_xstar(const Es1dConst &c, double x
   return Point64<ORDER>(__dmul_rn(wrap_fast(__fma_rn(c.hdt, v, x), c.L, err), c.inv_h), c.nc);
 }
 
-// The nodes' largest |amounts| of the current state's deposits to the scales (zero
-// before) of J1, parity par, and of J2 (v* is near v).
+// The nodes' largest |amounts| of the current state's deposits to the records (zero
+// before) of J1 and of J2 (v* is near v), the largest |v| to vmax of parity par.
 template <int ORDER>
 __global__ void __launch_bounds__(512, 2) mom_absmax_kernel(Es1dConst c, Es1dFp64Bufs b,
                                                             int par) {
   __shared__ unsigned W[kMomMaxNodes];
   clear_largest(W, c.nc);
   __syncthreads();
+  unsigned vm = 0;
   const int64_t end = chunk_end(c);
   for (int64_t p = blockIdx.x * c.chunk + threadIdx.x; p < end; p += blockDim.x) {
     const double v = b.v[p];
+    vm = max(vm, abs_hi(v));
     const int s = species_of(c, p);
     double A = v;
     if (!c.fold) A *= b.w ? c.q_h[s] * b.w[p] : c.qw_h[s];
     raise_largest(W + mom_xstar<ORDER>(c, b.x[p], v, b.err).i, abs_hi(A) >> 20);
   }
   __syncthreads();
-  flush_largest(W, b.amax + par * c.nc, c.nc);
-  flush_largest(W, b.amax + 2 * c.nc, c.nc);
-  flush_largest(W, b.amax + 3 * c.nc, c.nc);
+  flush_vmax(vm, b.vmax + par);
+  flush_largest(W, b.rec, c.nc);
+  flush_largest(W, b.rec + c.nc, c.nc);
+}
+// The first scale words (one block).
+__global__ void __launch_bounds__(512) mom_scales_kernel(Es1dConst c, Es1dFp64Bufs b, int par) {
+  __shared__ unsigned S[kMomMaxNodes + 2 * kMostReach];
+  for (int k = 0; k < 2; k++) {
+    ScaleMaker<>(b.words + k * (c.nc + 1), b.rec + k * c.nc, c.nc)
+        .make(S, node_reach(__ldcg(b.vmax + par), c.reach), 0);
+    __syncthreads();
+  }
 }
 
 // j^{n,*} of the current state (ESEC2 start-up and after a state change).
@@ -353,7 +368,7 @@ __global__ void __launch_bounds__(512, 2) mom_deposit_initial_kernel(Es1dConst c
   unsigned *T = m_.T, *W = m_.W;
   const int copies = c.copies;
   clear_fixed(T, 2 * nc * (ORDER + 1) * copies);
-  ScaleWords(b.amax + par * nc, nullptr, nc).store(W);
+  ScaleWords(b.words, nc + 1).store(W);
   __syncthreads();
   unsigned *Tl = T + (threadIdx.x & (copies - 1));
   const double scale = c.fold ? c.qw_h[0] : 1.0;
@@ -366,11 +381,11 @@ __global__ void __launch_bounds__(512, 2) mom_deposit_initial_kernel(Es1dConst c
     b.sds[p] = N.d;
     double A = v;
     if (!c.fold) A *= b.w ? c.q_h[s] * b.w[p] : c.qw_h[s];
-    add_moments<ORDER>(Tl + (size_t)N.i * 2 * (ORDER + 1) * copies, copies, W + N.i, nullptr, 0, N,
-                       A, scale, b.J1[par], &b.Jt[par], nc);
+    add_moments<ORDER>(Tl + (size_t)N.i * 2 * (ORDER + 1) * copies, copies, W + N.i, N, A, scale,
+                       b.J1[par], &b.Jt[par], nc);
   }
   __syncthreads();
-  flush_moments<ORDER>(T, W, copies, nc, scale, b.J1[par], &b.Jt[par]);
+  flush_moments<ORDER>(T, W, copies, nc, scale, b.J1[par], &b.Jt[par], ScaleRange(W[nc]));
 }
 
 template <typename F>
@@ -386,7 +401,7 @@ void dispatch_mom(const Es1dConst &c, F f) {
 
 size_t mom_smem(const Es1dConst &c, int copies, bool late) {
   const size_t words = (size_t)(c.order == 1 ? 2 : 4) + (size_t)(c.order + 1) * copies;
-  return sizeof(double) * (words * c.nc + (c.nc + 1) / 2 * 2) + (late ? 0 : sizeof(unsigned) * c.nc);
+  return sizeof(double) * (words * c.nc + (c.nc + 1) / 2 * 2) + (late ? 0 : sizeof(unsigned) * (c.nc + 1));
 }
 size_t mom_smem(const Es1dConst &c) { return mom_smem(c, c.copies, c.late); }
 
@@ -424,11 +439,12 @@ cudaError_t es1d_mom_prepare(const Es1dConst &c) {
   return e;
 }
 
-// (b.Jt and b.amax zero before) the deposits' scale and, for ESEC2, j^{n,*}
+// (b.Jt, b.vmax, b.words and b.rec zero before) the deposits' scale and, for ESEC2, j^{n,*}
 void es1d_mom_start(const Es1dConst &c, const Es1dFp64Bufs &b, int parity, LaunchShape ls,
                     cudaStream_t st) {
   (c.order == 1 ? mom_absmax_kernel<1> : mom_absmax_kernel<2>)
       <<<ls.grid, ls.block, 0, st>>>(c, b, parity);
+  mom_scales_kernel<<<1, 512, 0, st>>>(c, b, parity);
   if (c.scheme == 2)
     launch_dependent(c.order == 1 ? mom_deposit_initial_kernel<1> : mom_deposit_initial_kernel<2>,
                      ls, mom_smem(c), st, false, c, b, parity);

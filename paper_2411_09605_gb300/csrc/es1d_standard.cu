@@ -90,8 +90,7 @@ __device__ __forceinline__ void std_deposit(unsigned *Tl, unsigned *W, const Std
     add_unit_moments<ORDER>(q, c.copies, P, c.qw_h[0], b.rho, b.rho + c.n, c.n);
   } else {
     const double A = std_qw(c, b, s, p);
-    add_moments<ORDER>(q, c.copies, W + P.i, b.amaxn + P.i, c.decay & 2, P, A, 1.0, b.rho, b.rho + c.n,
-                       c.n);
+    add_moments<ORDER>(q, c.copies, W + P.i, P, A, 1.0, b.rho, b.rho + c.n, c.n);
   }
 }
 template <int ORDER, bool FOLD>
@@ -107,12 +106,13 @@ __global__ void __launch_bounds__(kFixedMaxThreads, 2) std_step_kernel(StdConst 
   unsigned *T = (unsigned *)(sm + (ORDER + 1) * n), *W = std_scales<ORDER, FOLD>(T, c);
   clear_fixed(T, 2 * (ORDER + 1) * n * copies);
   griddep_wait();
-  const ScaleWords words(b.amax, b.amaxn, FOLD ? 0 : n);
+  const ScaleWords words(b.words, FOLD ? 0 : n + 1);
   build_poly_std<ORDER>(sm, b.E, n, FOLD ? c.dt_qm[0] : 1.0);
   words.store(W);
   unsigned *Tl = T + (threadIdx.x & (copies - 1));
   __syncthreads();
   double ke = 0.0;
+  unsigned vm = 0;
   const int64_t end = chunk_end(c);
   for (int64_t p = blockIdx.x * c.chunk + threadIdx.x; p < end; p += blockDim.x) {
     const int s = FOLD ? 0 : species_of_std(c, p);
@@ -126,6 +126,7 @@ __global__ void __launch_bounds__(kFixedMaxThreads, 2) std_step_kernel(StdConst 
     const double x1 = wrap_fast(__fma_rn(c.dt, vn, x), c.L, b.err);
     b.x[p] = x1;
     b.v[p] = vn;
+    if (!FOLD) vm = max(vm, abs_hi(vn));
     const Point64<ORDER> P(__dmul_rn(x1, c.inv_h), n);
     b.si[p] = P.i;   // the next step gathers there
     b.sd[p] = P.d;
@@ -133,24 +134,35 @@ __global__ void __launch_bounds__(kFixedMaxThreads, 2) std_step_kernel(StdConst 
   }
   griddep_launch_dependents();
   if (!isfinite(ke)) atomicOr(b.err, kErrNonfinite);
+  if (!FOLD) flush_vmax(vm, b.vmax);
   const double kb = block_sum_narrow(ke, red);   // (its barriers order the tile's sums)
   if (threadIdx.x == 0) b.ke_part[blockIdx.x] = FOLD ? 0.5 * c.half_m[0] * c.w0[0] * kb : kb;
-  flush_moments<ORDER, 1, !FOLD>(T, W, copies, n, FOLD ? c.qw_h[0] : 1.0, b.rho, b.rho + n);
+  if (!FOLD) flush_new(W, b.rec, n);
+  flush_moments<ORDER, 1, !FOLD>(T, W, copies, n, FOLD ? c.qw_h[0] : 1.0, b.rho, b.rho + n,
+                                 FOLD ? ScaleRange(0, 0) : ScaleRange(W[n]));
 }
 
-// The nodes' largest |charges| to amax and amaxn (zero before).
+// The nodes' largest |charges| to the records (zero before).
 template <int ORDER>
 __global__ void __launch_bounds__(kFixedMaxThreads, 2) std_amax_kernel(StdConst c, StdBufs b) {
   __shared__ unsigned W[kStdMaxNodes];
   clear_largest(W, c.n);
   __syncthreads();
+  unsigned vm = 0;
   const int64_t end = chunk_end(c);
-  for (int64_t p = blockIdx.x * c.chunk + threadIdx.x; p < end; p += blockDim.x)
+  for (int64_t p = blockIdx.x * c.chunk + threadIdx.x; p < end; p += blockDim.x) {
+    vm = max(vm, abs_hi(b.v[p]));
     raise_largest(W + Point64<ORDER>(__dmul_rn(b.x[p], c.inv_h), c.n).i,
                   abs_hi(std_qw(c, b, species_of_std(c, p), p)) >> 20);
+  }
+  flush_vmax(vm, b.vmax);
   __syncthreads();
-  flush_largest(W, b.amax, c.n);
-  flush_largest(W, b.amaxn, c.n);
+  flush_largest(W, b.rec, c.n);
+}
+// The first scale words (one block).
+__global__ void __launch_bounds__(512) std_scales_kernel(StdConst c, StdBufs b) {
+  __shared__ unsigned S[kStdMaxNodes + 2 * kMostReach];
+  ScaleMaker<>(b.words, b.rec, c.n).make(S, node_reach(__ldcg(b.vmax), c.reach), 0);
 }
 
 // The charge and the points of x^0.
@@ -160,7 +172,7 @@ __global__ void __launch_bounds__(kFixedMaxThreads, 2) std_charge_kernel(StdCons
   const int n = c.n, copies = c.copies;
   unsigned *T = (unsigned *)(sm + (ORDER + 1) * n), *W = std_scales<ORDER, FOLD>(T, c);
   clear_fixed(T, 2 * (ORDER + 1) * n * copies);
-  ScaleWords(b.amax, b.amaxn, FOLD ? 0 : n).store(W);
+  ScaleWords(b.words, FOLD ? 0 : n + 1).store(W);
   __syncthreads();
   unsigned *Tl = T + (threadIdx.x & (copies - 1));
   const int64_t end = chunk_end(c);
@@ -172,7 +184,9 @@ __global__ void __launch_bounds__(kFixedMaxThreads, 2) std_charge_kernel(StdCons
     std_deposit<ORDER, FOLD>(Tl, W, c, b, s, p, P);
   }
   __syncthreads();
-  flush_moments<ORDER, 1, !FOLD>(T, W, copies, n, FOLD ? c.qw_h[0] : 1.0, b.rho, b.rho + n);
+  if (!FOLD) flush_new(W, b.rec, n);
+  flush_moments<ORDER, 1, !FOLD>(T, W, copies, n, FOLD ? c.qw_h[0] : 1.0, b.rho, b.rho + n,
+                                 FOLD ? ScaleRange(0, 0) : ScaleRange(W[n]));
 }
 
 // E^{n+1} into En from rho [n] and its total rho[n]: block 0 writes TE^n (slot >= 0)
@@ -190,10 +204,13 @@ __global__ void __launch_bounds__(kStdSolveThreads) std_solve_kernel(StdConst c,
   griddep_launch_dependents();
   if (blockIdx.x == 0) {
     for (int i = threadIdx.x; i <= n; i += blockDim.x) b.rhon[i] = 0.0;
-    // (the last markers' scales have been used: their place takes the next markers'
-    // largest charges)
-    for (int i = threadIdx.x; i < n && !c.fold; i += blockDim.x)
-      b.amax[i] = scale_start(b.amaxn[i], c.decay);
+    // the next markers' scales, from what the last ones recorded
+    if (!c.fold) {
+      ScaleMaker<>(b.words, b.rec, n)
+          .make((unsigned *)sm, node_reach(__ldcg(b.vmax), c.reach), c.decay);
+      __syncthreads();
+      if (threadIdx.x == 0) *b.vmax = 0u;
+    }
     if (slot < 0) return;
     double t = 0.0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) t = fma(0.5 * c.h * b.E[i], b.E[i], t);
@@ -273,7 +290,7 @@ __global__ void std_response_kernel(StdConst c, StdBufs b) {
 
 size_t std_smem(const StdConst &c, int copies) {
   return sizeof(double) * (size_t)(c.order + 1) * (1 + (size_t)copies) * c.n +
-         (c.fold ? 0 : sizeof(unsigned) * c.n);
+         (c.fold ? 0 : sizeof(unsigned) * (c.n + 1));
 }
 size_t std_solve_smem(const StdConst &c) { return sizeof(double) * 2 * (size_t)c.n; }
 
@@ -332,10 +349,12 @@ void std_field(const StdConst &c, const StdBufs &b, int slot, LaunchShape lp, cu
   std_solve(c, b, slot, lp, st, true);
 }
 
-// (rho, rhon, amax and amaxn zero before) the charge of x^0 and E^0 into b.En.
+// (rho, rhon, vmax, words and rec zero before) the charge of x^0 and E^0 into b.En.
 void std_start_field(const StdConst &c, const StdBufs &b, LaunchShape lp, cudaStream_t st) {
-  if (!c.fold)
+  if (!c.fold) {
     (c.order == 1 ? std_amax_kernel<1> : std_amax_kernel<2>)<<<lp.grid, lp.block, 0, st>>>(c, b);
+    std_scales_kernel<<<1, 512, 0, st>>>(c, b);
+  }
   dispatch_std(c, [&](auto O, auto F) {
     std_charge_kernel<decltype(O)::value, decltype(F)::value>
         <<<lp.grid, lp.block, std_smem(c, c.copies), st>>>(c, b);

@@ -673,8 +673,14 @@ int init_mixed(pic_handle *h, bool solve_e0) {
   return PIC_OK;
 }
 
-// The moment passes' totals and largest amounts, in doubles.
-size_t mom_scalar_words(const Es1dConst &c) { return 4 + 2 * (size_t)c.nc; }
+// The moment passes' totals Jt [4], largest speeds, scale words and records, in doubles.
+size_t mom_scalar_words(const Es1dConst &c) { return 6 + 2 * (size_t)c.nc; }
+void mom_scalars(const Es1dConst &c, Es1dFp64Bufs &b, double *at) {
+  b.Jt = at;
+  b.vmax = (unsigned *)(at + 4);
+  b.words = b.vmax + 2;
+  b.rec = b.words + 2 * (c.nc + 1);
+}
 
 // What the first step of an FP64 1D state needs beside its zero currents:
 // j^{n,*} (ESEC2), and the moment passes' deposit scales.
@@ -716,6 +722,7 @@ int init_es1d(pic_handle *h, const pic_species *species, const double *E0) {
     c.hdt_qm[s] = 0.5 * c.dt * c.qm[s];
   }
   c.hdt = 0.5 * c.dt;
+  c.reach = (float)(c.dt * c.inv_h);
   c.inv_nc = 1.0 / c.nc;
   c.fold = h->nsp == 1 && !h->weighted;
   h->mom = !h->mixed && es1d_fp64_use_moments(c);
@@ -743,7 +750,7 @@ int init_es1d(pic_handle *h, const pic_species *species, const double *E0) {
   b.sd = nullptr;
   b.sds = nullptr;
   b.Jt = nullptr;
-  b.amax = nullptr;
+  b.vmax = b.words = b.rec = nullptr;
   // a point's shape between the passes: its node and its offset (the moment
   // passes) or weights
   const size_t nsh = (size_t)(h->mom ? 1 : c.order + 1) * h->N;
@@ -755,9 +762,9 @@ int init_es1d(pic_handle *h, const pic_species *species, const double *E0) {
       ((rc = h->alloc(h->mom ? &b.sds : &b.sws, nsh)) || (rc = h->alloc(&b.sis, h->N))))
     return rc;
   if (h->mom) {
-    // Jt [4] and amax [4][nc] in one block, cleared together
+    // in one block, cleared together
     if ((rc = h->alloc(&b.Jt, mom_scalar_words(c)))) return rc;
-    b.amax = (unsigned *)(b.Jt + 4);
+    mom_scalars(c, b, b.Jt);
     CUDA_TRY(cudaMemsetAsync(b.Jt, 0, sizeof(double) * mom_scalar_words(c), h->st));
   }
   b.w = nullptr;
@@ -1147,15 +1154,13 @@ int restart_std(pic_handle *h) {
   CUDA_TRY(cudaGetLastError());
   CUDA_TRY(cudaMemsetAsync(b.rho, 0, sizeof(double) * (h->cs.n + 1), h->st));
   CUDA_TRY(cudaMemsetAsync(b.rhon, 0, sizeof(double) * (h->cs.n + 1), h->st));
-  CUDA_TRY(cudaMemsetAsync(b.amax, 0, sizeof(unsigned) * h->cs.n, h->st));
-  CUDA_TRY(cudaMemsetAsync(b.amaxn, 0, sizeof(unsigned) * h->cs.n, h->st));
+  CUDA_TRY(cudaMemsetAsync(b.vmax, 0, sizeof(unsigned) * (2 + 2 * (size_t)h->cs.n), h->st));
   std_start_field(h->cs, b, h->lsd, h->st);
   std::swap(b.E, b.En);
   std::swap(b.rho, b.rhon);
-  std::swap(b.amax, b.amaxn);
   std_kick_back(h->cs, b, h->lsd, h->st);
   CUDA_TRY(cudaGetLastError());
-  h->launches += 4 + !h->cs.fold;
+  h->launches += 4 + 2 * !h->cs.fold;
   return check_flags(h, "pic_init/pic_set_*");
 }
 
@@ -1186,6 +1191,7 @@ int init_std(pic_handle *h, const pic_species *species) {
   }
   for (int s = h->nsp; s < kMaxSpecies; s++) c.sp_end[s] = h->N;
   c.inv_n = 1.0 / c.n;
+  c.reach = (float)(c.dt * c.inv_h);
   for (int s = 0; s < h->nsp; s++) c.dt_qm[s] = c.dt * c.qm[s];
   c.fold = h->nsp == 1 && !h->weighted;
   h->lsd = std_shape(c, h->nsm);
@@ -1199,12 +1205,14 @@ int init_std(pic_handle *h, const pic_species *species) {
   if ((rc = h->alloc(&b.sd, h->N)) || (rc = h->alloc(&b.si, h->N)) || (rc = h->alloc(&b.E, n)) ||
       (rc = h->alloc(&b.En, n)) || (rc = h->alloc(&b.rho, n + 1)) ||
       (rc = h->alloc(&b.rhon, n + 1)) || (rc = h->alloc(&b.resp, n)) ||
-      (rc = h->alloc(&b.amax, n)) || (rc = h->alloc(&b.amaxn, n)) ||
+      (rc = h->alloc(&b.vmax, 2 + 2 * n)) ||
       (rc = h->alloc(&b.ke_part, (size_t)h->lsd.grid)) ||
       (rc = h->alloc(&b.fallback, kStepsCap)) || (rc = h->alloc(&b.te, kStepsCap)) ||
       (rc = h->alloc(&b.err, 1)) || (rc = h->alloc(&h->ids, h->N)) ||
       (rc = h->alloc(&h->std_part, (size_t)h->lsd.grid * h->nsp + 1)))
     return rc;
+  b.words = b.vmax + 1;   // cleared together
+  b.rec = b.words + n + 1;
   h->b1.err = b.err;
   h->b1.fallback = b.fallback;
   h->b1.te = b.te;
@@ -1257,9 +1265,9 @@ int restart_em1d(pic_handle *h, bool markers_changed = true) {
     em1m_start(h->c1e, b, h->c1m, mb, h->le, h->st);
     h->launches += 1 + (markers_changed ? 2 : 1) + 2 * (h->c1e.scheme == 2);
   } else {
-    CUDA_TRY(cudaMemsetAsync(b.amax, 0, sizeof(unsigned) * 8 * h->c1e.n, h->st));
+    CUDA_TRY(cudaMemsetAsync(b.vmax, 0, sizeof(unsigned) * (2 + 8 * h->c1e.n), h->st));
     em1d_start(h->c1e, b, h->le, h->st);
-    h->launches += 3 + (h->c1e.scheme == 2);
+    h->launches += 4 + (h->c1e.scheme == 2);
   }
   CUDA_TRY(cudaGetLastError());
   return check_flags(h, "pic_init/pic_set_*");
@@ -1373,6 +1381,7 @@ int init_em1d(pic_handle *h, const pic_species *species, const double *E0, const
   }
   for (int s = h->nsp; s < kMaxSpecies; s++) c.sp_end[s] = h->N;
   c.hdt = 0.5 * c.dt;
+  c.reach = (float)(c.dt * c.inv_h);
   for (int s = 0; s < h->nsp; s++) {
     c.dt_qm[s] = c.dt * c.qm[s];
     c.hdt_qm[s] = 0.5 * c.dt * c.qm[s];
@@ -1406,10 +1415,14 @@ int init_em1d(pic_handle *h, const pic_species *species, const double *E0, const
   // ESEC2, the next y* from pass E to pass C
   b.sd = b.sds = nullptr;
   b.si = b.sis = nullptr;
-  b.amax = nullptr;
+  b.vmax = b.words = b.rec = nullptr;
   if (!h->mixed && ((rc = h->alloc(&b.sd, h->N)) || (rc = h->alloc(&b.si, h->N)) ||
-                    (rc = h->alloc(&b.amax, 8 * n))))
+                    (rc = h->alloc(&b.vmax, 2 + 8 * n))))
     return rc;
+  if (b.vmax) {   // cleared together
+    b.words = b.vmax + 2;
+    b.rec = b.words + 4 * n;
+  }
   if (!h->mixed && cfg.scheme == 2 &&
       ((rc = h->alloc(&b.sds, h->N)) || (rc = h->alloc(&b.sis, h->N))))
     return rc;
@@ -1686,7 +1699,6 @@ int pic_step_async(pic_handle *h, int nsteps) {
     CUDA_TRY(h->timed_launch(4, [&] { std_field(h->cs, h->bs, slot, h->lsd, h->st); }));
     std::swap(h->bs.E, h->bs.En);
     std::swap(h->bs.rho, h->bs.rhon);
-    std::swap(h->bs.amax, h->bs.amaxn);
     h->launches += 2;
     h->steps_done++;
     h->pending++;
@@ -2350,8 +2362,7 @@ int grad_rerun_mom(pic_handle *h, int seg, int s0, int s1, bool all, double *sca
   const int64_t at = h->steps_done;
   GradSwing w(h);
   Es1dFp64Bufs &b = h->b1;
-  b.Jt = scal;
-  b.amax = (unsigned *)(scal + 4);
+  mom_scalars(h->c1, b, scal);
   b.J2[0] = J2;
   b.J2[1] = J2 + nc;
   if (b.sds) {
@@ -2386,14 +2397,15 @@ int grad_backward_mom(pic_handle *h, const double *Ebar, const double *xbar, con
   const size_t N = (size_t)h->N, nc = (size_t)h->c1.nc, rec = grad_rec_words(h);
   const int seglen = std::min(g.every, g.nsteps);
   const size_t words = es1d_rev_table_words(h->c1);
-  const size_t kScal = 5 + mom_scalar_words(h->c1) + 3 * nc;
+  const size_t kScal = 6 + mom_scalar_words(h->c1) + 3 * nc;
   if (!g.grid) CUDA_TRY(cudaMalloc(&g.grid, sizeof(double) * (7 * nc + kScal)));
   if (!g.mk) CUDA_TRY(cudaMalloc(&g.mk, sizeof(double) * 9 * N + 16));
   CUDA_TRY(grad_room(&g.seg, &g.seg_cap, (seglen + 1) * rec));
   CUDA_TRY(grad_room(&g.tab, &g.tab_cap, seglen * words));
   CUDA_TRY(es1d_rev_prepare(h->c1));
   CUDA_TRY(cudaMemsetAsync(g.grid, 0, sizeof(double) * (7 * nc + kScal), h->st));
-  // scalars: the re-run's passes', five sums and the nodes' six words of the reverse
+  // scalars: the re-run's passes', five sums, two speeds and the nodes' six words of the
+  // reverse
   double *scal = g.grid + 7 * nc, *mk = g.mk;
   Es1dRevBufs r{};
   r.w = h->b1.w;
@@ -2406,7 +2418,8 @@ int grad_backward_mom(pic_handle *h, const double *Ebar, const double *xbar, con
   double *J2 = g.grid + 5 * nc;
   r.gtot = scal + mom_scalar_words(h->c1);
   r.tot = r.gtot + 1;
-  r.mx = (unsigned *)(r.gtot + 5);
+  r.umax = (unsigned *)(r.gtot + 5);
+  r.mx = r.umax + 2;
   r.xb = mk;
   r.vb = mk + N;
   r.wb = mk + 2 * N;
@@ -2435,6 +2448,7 @@ int grad_backward_mom(pic_handle *h, const double *Ebar, const double *xbar, con
   int par = 0;
   if (r.vin) {
     r.x = h->b1.x;
+    r.v = h->b1.v;
     es1d_rev_start(h->c1, r, par, h->lmom, h->st);
     CUDA_TRY(cudaGetLastError());
     h->launches += 1;

@@ -61,6 +61,7 @@ struct Es1dConst {
   int fold;
   int copies;                    // tile copies of a block (a power of two)
   int late;                      // the nodes' scale words take the place of the field
+  float reach;                   // dt / h
   int decay;                     // whether the nodes' scales fall (scale_decay)
   int64_t chunk;                 // markers of a block
   double inv_nc;                 // 1 / nc
@@ -236,6 +237,7 @@ struct Em1dConst {
   int nsp;
   int copies;       // FP64 passes: copies of the shared current tile (power of two, <= 32)
   int decay;        // FP64 passes: whether the nodes' scales fall (scale_decay)
+  float reach;      // dt / h
   int fold;         // one uniformly weighted species: its factors go to tables and sums
   int64_t chunk;    // FP64 passes: markers of a block
   int direct;       // 1: the direct field solve (n <= kEm1DirectNodes), a service block first
@@ -257,8 +259,9 @@ struct Em1dBufs {
   int *si;                   // [N] the node (pass C -> pass E)
   double *sds;               // ESEC2: the next step's y* (pass E or the initial deposit
   int *sis;                  // -> pass C), as sd / si; null: formed again
-  unsigned *amax;            // [2][2][n][2] exponents of the nodes' largest amounts in J1 and J2:
-                             // of the last pass and of the present one
+  unsigned *words;           // [2][n][2] the nodes' scale words (fixed_moments.cuh) of J1, J2 and
+  unsigned *rec;             // [2][n][2] the larger amounts recorded since
+  unsigned *vmax;            // [2] the largest |vy| (high word): of the last step, of this one
   double *E, *En;            // E^n, E^{n+1}: [2][n] (Ex, Ey); swapped after each step
   double *B, *Bn;            // Bz^n, Bz^{n+1}: [n]
   double *Es, *Bs;           // E*, B* of the half step
@@ -285,6 +288,7 @@ struct StdConst {
   int nsp;
   int copies;       // copies of the shared charge tile (power of two, <= 32)
   int decay;        // whether the nodes' scales fall (scale_decay)
+  float reach;      // dt / h
   int fold;         // one uniformly weighted species: its factors go to tables and sums
   int64_t chunk;    // markers of a block
   int passes;       // 1-2-1 filter passes on the charge
@@ -307,8 +311,9 @@ struct StdBufs {
   double *rho, *rhon;    // [n + 1] charge of the next positions and its total; the other
                          // buffer is cleared meanwhile, swapped after each step
   double *resp;          // [n] E of a unit charge at node 0
-  unsigned *amax, *amaxn;   // [n] exponents of the nodes' largest charges (several species,
-                            // weights) of the last markers and the next; swapped as rho
+  unsigned *words, *rec;    // [n + 1] the nodes' scale words (fixed_moments.cuh; several species,
+                            // weights) and their range, [n] the larger charges recorded since
+  unsigned *vmax;           // [1] the largest |v| (high word)
   double *ke_part;       // [particle blocks]
   unsigned long long *fallback;
   double *te;
@@ -406,7 +411,10 @@ struct Es1dFp64Bufs {
   double *sd, *sds;         // moment passes: [N] the offset from node si (sis) in
                             // place of the weights sw (sws); null otherwise
   double *Jt;               // moment passes: totals of J1[0], J1[1], J2[0], J2[1]
-  unsigned *amax;           // and [4][nc] the exponents of the nodes' largest amounts in them
+  unsigned *words;          // and [2][nc + 1] the nodes' scale words (fixed_moments.cuh) of J1, J2
+                            // and their range,
+  unsigned *rec;            // [2][nc] the larger amounts recorded since
+  unsigned *vmax;           // and [2] the largest |v| (high word) by step parity
   double *E[2];             // ping-pong E^n / E^{n+1}
   double *J1[2];            // j^{n,*} (ESEC2), indexed by step parity
   double *J2[2];            // j^{*,n+1/2}
@@ -456,12 +464,10 @@ cudaError_t allow_shared(K *kern, size_t bytes) {
                               room);
 }
 
-// Whether a step (bit 0) and the one before it (bit 1) let the scales of the fixed-point
-// deposits fall by one exponent (fixed_moments.cuh).
+// Whether a step lets the scales of the fixed-point deposits fall by one exponent
+// (fixed_moments.cuh).
 constexpr int kScaleSteps = 8;
-inline int scale_decay(int64_t step) {
-  return (step % kScaleSteps == 0) | (step % kScaleSteps == 1) << 1;
-}
+inline int scale_decay(int64_t step) { return step % kScaleSteps == 0; }
 
 // Sets the message returned by pic_last_error (pic_api.cu).
 void set_last_error(const std::string &msg);
@@ -491,6 +497,7 @@ struct Es1dRevBufs {
   double *Hb[2], *Es[2];    // [nc] adjoints of E^{n+1/2} and E* by step parity
   double *tot;              // [2][2] their totals
   unsigned *mx;             // [2][3][nc] exponents of the nodes' largest amounts
+  unsigned *umax;           // [2] the largest |v*| (high word)
   double *xb, *vb, *wb;     // [N] adjoints of the markers (x in cells)
   double *ub, *yb, *u, *ap, *dy;   // [N] marker scratch
   long long *D;
