@@ -39,13 +39,14 @@
 // All kernels are programmatic dependent launches: the tile is cleared before
 // the wait for the previous kernel.
 //
-// Measured (2^23 markers, 512 nodes, order 2, ESEC2), against the general passes
-// / with shared FP64 atomics in place of the fixed-point sums / now: pass C 598 /
-// 221 / 117 us (warp instructions on the FP64 pipe per 32 markers 32.6 / 13.4 /
-// 6.5), pass E 986 / 387 / 240 us (56.8 / 24.6 / 14.8); the pipe is 78 and 85%
-// busy.  20,000 markers on 64 nodes: 36.6 / 11.8 / 11.4 us a step, bound by the
-// launches' serial parts (loads, tables, flush); 50 steps and their results 557 us
-// with a thread's first marker loaded after the table is built, 540 before it.
+// Measured (2^23 markers, 512 nodes, order 2, ESEC2), with the general passes / with
+// shared FP64 atomics in place of the fixed-point sums / with those and one unit for the
+// grid / now, with a unit a node: pass C 598 / 221 / 119 / 122 us (warp instructions on
+// the FP64 pipe per 32 markers 32.6 / 13.4 / 6.5 / 6.8), pass E 986 / 387 / 244 / 246 us
+// (56.8 / 24.6 / 14.8 / 15.2).  20,000 markers on 64 nodes: 36.6 / 11.8 / 10.5 / 11.1 us
+// a step, bound by the launches' serial parts (loads, tables, flush); 1,000 on 1792 nodes
+// 43 / - / 21 / 28, the flush; 50 steps and their results 557 us with a thread's first
+// marker loaded after the table is built, 540 before it.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -2866,6 +2866,7 @@ std::vector<int> batch_blocks(const std::vector<pic_handle *> &runs, double targ
 // run.
 std::vector<int> batch_items(const std::vector<pic_handle *> &runs, double lo, double hi,
                              int threads, std::vector<BatchItem> &items) {
+  // (blocks an SM: the kernels' launch bounds)
   const int places = runs[0]->nsm * (threads == 1024 ? 1 : 3);
   double groups = 0.0;
   for (const pic_handle *h : runs) groups += (double)((h->N + 3) / 4);
