@@ -45,7 +45,7 @@
 // the FP64 pipe per 32 markers 32.6 / 13.4 / 6.5 / 6.8), pass E 986 / 387 / 244 / 246 us
 // (56.8 / 24.6 / 14.8 / 15.2).  20,000 markers on 64 nodes: 36.6 / 11.8 / 10.5 / 11.1 us
 // a step, bound by the launches' serial parts (loads, tables, flush); 1,000 on 1792 nodes
-// 43 / - / 21 / 28, the flush; 50 steps and their results 557 us with a thread's first
+// 43 / - / 21 / 29, the flush; 50 steps and their results 557 us with a thread's first
 // marker loaded after the table is built, 540 before it.
 #include <cuda_runtime.h>
 
@@ -135,12 +135,13 @@ __global__ void __launch_bounds__(512, 2) mom_pass_c_kernel(Es1dConst c, Es1dFp6
     }
     if (threadIdx.x == 0) b.vmax[par ^ 1] = 0u;
     // pass E's scales, from what the pass E before recorded (all loads first)
-    const ScaleMaker<> scales(b.words, b.rec, SCHEME == 2 ? nc : 0);
+    const ScaleMaker<> scales(b.words, b.rec, b.storm, SCHEME == 2 ? nc : 0);
     const unsigned vmax = __ldcg(b.vmax + par);
     double s = 0.0;
     if (prev_slot >= 0)
       for (int i = threadIdx.x; i < nblk; i += blockDim.x) s += b.ke_part[i];
-    if (SCHEME == 2) scales.make((unsigned *)sm, node_reach(vmax, c.reach), c.decay);
+    if (SCHEME == 2)
+      scales.make((unsigned *)sm, node_reach(vmax, c.reach), c.decay, c.n_total);
     if (prev_slot >= 0) {
       const double t = block_sum_narrow(s, red);
       if (threadIdx.x == 0) {
@@ -192,12 +193,12 @@ __global__ void __launch_bounds__(512, 2) mom_pass_c_kernel(Es1dConst c, Es1dFp6
     b.sd[p] = H.d;
     double A = vs;
     if (!FOLD) A *= b.w ? c.q_h[s] * b.w[p] : c.qw_h[s];
-    add_moments<ORDER>(Tl + (size_t)H.i * 2 * (ORDER + 1) * copies, copies, W + H.i, H, A, scale,
+    add_moments<ORDER>(Tl + (size_t)H.i * 2 * (ORDER + 1) * copies, copies, W + H.i, W + nc + 1, H, A, scale,
                        b.J2[par], &b.Jt[2 + par], nc);
   }
   griddep_launch_dependents();
   __syncthreads();
-  flush_new(W, b.rec + nc, nc);
+  flush_new(W, b.rec + nc, nc, W + nc + 1, b.storm + 2);
   flush_moments<ORDER>(T, W, copies, nc, scale, b.J2[par], &b.Jt[2 + par], ScaleRange(W[nc]));
 }
 
@@ -212,7 +213,7 @@ __global__ void __launch_bounds__(512, 2) mom_pass_e_kernel(Es1dConst c, Es1dFp6
   if ((int)blockIdx.x == nblk) {   // service block: E^{n+1}, W_E, the cleared J2
     griddep_wait();
     griddep_launch_dependents();
-    const ScaleMaker<> scales(b.words + nc + 1, b.rec + nc, nc);
+    const ScaleMaker<> scales(b.words + nc + 1, b.rec + nc, b.storm + 2, nc);
     const unsigned vmax = __ldcg(b.vmax + par);
     const double mean = c.remove_mean ? b.Jt[2 + par] * c.inv_nc : 0.0;
     double we = 0.0;
@@ -228,7 +229,7 @@ __global__ void __launch_bounds__(512, 2) mom_pass_e_kernel(Es1dConst c, Es1dFp6
       b.Jt[2 + (par ^ 1)] = 0.0;
     }
     // the next pass C's scales, from what the last one recorded
-    scales.make((unsigned *)sm, node_reach(vmax, c.reach), c.decay);
+    scales.make((unsigned *)sm, node_reach(vmax, c.reach), c.decay, c.n_total);
     return;
   }
   const MomShared<ORDER> m_(c, sm);
@@ -302,7 +303,7 @@ __global__ void __launch_bounds__(512, 2) mom_pass_e_kernel(Es1dConst c, Es1dFp6
       b.sds[p] = N.d;
       double A = vn;
       if (!FOLD) A *= b.w ? c.q_h[s] * wp : c.qw_h[s];
-      add_moments<ORDER>(Tl + (size_t)N.i * 2 * (ORDER + 1) * copies, copies, W + N.i, N, A, scale,
+      add_moments<ORDER>(Tl + (size_t)N.i * 2 * (ORDER + 1) * copies, copies, W + N.i, W + nc + 1, N, A, scale,
                          b.J1[par ^ 1], &b.Jt[par ^ 1], nc);
     }
   }
@@ -313,7 +314,7 @@ __global__ void __launch_bounds__(512, 2) mom_pass_e_kernel(Es1dConst c, Es1dFp6
   const double t = block_sum_narrow(ke, red);   // (its barriers order the tile before the flush)
   if (threadIdx.x == 0) b.ke_part[blockIdx.x] = FOLD ? c.half_mw[0] * t : t;
   if (SCHEME == 2) {
-    flush_new(W, b.rec, nc);
+    flush_new(W, b.rec, nc, W + nc + 1, b.storm);
     flush_moments<ORDER>(T, W, copies, nc, scale, b.J1[par ^ 1], &b.Jt[par ^ 1],
                          ScaleRange(W[nc]));
   }
@@ -353,8 +354,8 @@ __global__ void __launch_bounds__(512, 2) mom_absmax_kernel(Es1dConst c, Es1dFp6
 __global__ void __launch_bounds__(512) mom_scales_kernel(Es1dConst c, Es1dFp64Bufs b, int par) {
   __shared__ unsigned S[kMomMaxNodes + 2 * kMostReach];
   for (int k = 0; k < 2; k++) {
-    ScaleMaker<>(b.words + k * (c.nc + 1), b.rec + k * c.nc, c.nc)
-        .make(S, node_reach(__ldcg(b.vmax + par), c.reach), 0);
+    ScaleMaker<>(b.words + k * (c.nc + 1), b.rec + k * c.nc, b.storm + 2 * k, c.nc)
+        .make(S, node_reach(__ldcg(b.vmax + par), c.reach), 0, c.n_total);
     __syncthreads();
   }
 }
@@ -382,7 +383,7 @@ __global__ void __launch_bounds__(512, 2) mom_deposit_initial_kernel(Es1dConst c
     b.sds[p] = N.d;
     double A = v;
     if (!c.fold) A *= b.w ? c.q_h[s] * b.w[p] : c.qw_h[s];
-    add_moments<ORDER>(Tl + (size_t)N.i * 2 * (ORDER + 1) * copies, copies, W + N.i, N, A, scale,
+    add_moments<ORDER>(Tl + (size_t)N.i * 2 * (ORDER + 1) * copies, copies, W + N.i, W + nc + 1, N, A, scale,
                        b.J1[par], &b.Jt[par], nc);
   }
   __syncthreads();
@@ -402,7 +403,7 @@ void dispatch_mom(const Es1dConst &c, F f) {
 
 size_t mom_smem(const Es1dConst &c, int copies, bool late) {
   const size_t words = (size_t)(c.order == 1 ? 2 : 4) + (size_t)(c.order + 1) * copies;
-  return sizeof(double) * (words * c.nc + (c.nc + 1) / 2 * 2) + (late ? 0 : sizeof(unsigned) * (c.nc + 1));
+  return sizeof(double) * (words * c.nc + (c.nc + 1) / 2 * 2) + (late ? 0 : sizeof(unsigned) * (c.nc + 2));
 }
 size_t mom_smem(const Es1dConst &c) { return mom_smem(c, c.copies, c.late); }
 

@@ -90,7 +90,7 @@ __device__ __forceinline__ void std_deposit(unsigned *Tl, unsigned *W, const Std
     add_unit_moments<ORDER>(q, c.copies, P, c.qw_h[0], b.rho, b.rho + c.n, c.n);
   } else {
     const double A = std_qw(c, b, s, p);
-    add_moments<ORDER>(q, c.copies, W + P.i, P, A, 1.0, b.rho, b.rho + c.n, c.n);
+    add_moments<ORDER>(q, c.copies, W + P.i, W + c.n + 1, P, A, 1.0, b.rho, b.rho + c.n, c.n);
   }
 }
 template <int ORDER, bool FOLD>
@@ -106,9 +106,9 @@ __global__ void __launch_bounds__(kFixedMaxThreads, 2) std_step_kernel(StdConst 
   unsigned *T = (unsigned *)(sm + (ORDER + 1) * n), *W = std_scales<ORDER, FOLD>(T, c);
   clear_fixed(T, 2 * (ORDER + 1) * n * copies);
   griddep_wait();
-  const ScaleWords words(b.words, FOLD ? 0 : n + 1);
+  const ScaleWords words(b.words, FOLD ? 0 : n + 1);   // (W null: not stored)
   build_poly_std<ORDER>(sm, b.E, n, FOLD ? c.dt_qm[0] : 1.0);
-  words.store(W);
+  if (!FOLD) words.store(W);
   unsigned *Tl = T + (threadIdx.x & (copies - 1));
   __syncthreads();
   double ke = 0.0;
@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(kFixedMaxThreads, 2) std_step_kernel(StdConst 
   if (!FOLD) flush_vmax(vm, b.vmax);
   const double kb = block_sum_narrow(ke, red);   // (its barriers order the tile's sums)
   if (threadIdx.x == 0) b.ke_part[blockIdx.x] = FOLD ? 0.5 * c.half_m[0] * c.w0[0] * kb : kb;
-  if (!FOLD) flush_new(W, b.rec, n);
+  if (!FOLD) flush_new(W, b.rec, n, W + n + 1, b.storm);
   flush_moments<ORDER, 1, !FOLD>(T, W, copies, n, FOLD ? c.qw_h[0] : 1.0, b.rho, b.rho + n,
                                  FOLD ? ScaleRange(0, 0) : ScaleRange(W[n]));
 }
@@ -162,7 +162,8 @@ __global__ void __launch_bounds__(kFixedMaxThreads, 2) std_amax_kernel(StdConst 
 // The first scale words (one block).
 __global__ void __launch_bounds__(512) std_scales_kernel(StdConst c, StdBufs b) {
   __shared__ unsigned S[kStdMaxNodes + 2 * kMostReach];
-  ScaleMaker<>(b.words, b.rec, c.n).make(S, node_reach(__ldcg(b.vmax), c.reach), 0);
+  ScaleMaker<>(b.words, b.rec, b.storm, c.n)
+      .make(S, node_reach(__ldcg(b.vmax), c.reach), 0, c.n_total);
 }
 
 // The charge and the points of x^0.
@@ -172,7 +173,7 @@ __global__ void __launch_bounds__(kFixedMaxThreads, 2) std_charge_kernel(StdCons
   const int n = c.n, copies = c.copies;
   unsigned *T = (unsigned *)(sm + (ORDER + 1) * n), *W = std_scales<ORDER, FOLD>(T, c);
   clear_fixed(T, 2 * (ORDER + 1) * n * copies);
-  ScaleWords(b.words, FOLD ? 0 : n + 1).store(W);
+  if (!FOLD) ScaleWords(b.words, n + 1).store(W);
   __syncthreads();
   unsigned *Tl = T + (threadIdx.x & (copies - 1));
   const int64_t end = chunk_end(c);
@@ -184,7 +185,7 @@ __global__ void __launch_bounds__(kFixedMaxThreads, 2) std_charge_kernel(StdCons
     std_deposit<ORDER, FOLD>(Tl, W, c, b, s, p, P);
   }
   __syncthreads();
-  if (!FOLD) flush_new(W, b.rec, n);
+  if (!FOLD) flush_new(W, b.rec, n, W + n + 1, b.storm);
   flush_moments<ORDER, 1, !FOLD>(T, W, copies, n, FOLD ? c.qw_h[0] : 1.0, b.rho, b.rho + n,
                                  FOLD ? ScaleRange(0, 0) : ScaleRange(W[n]));
 }
@@ -206,8 +207,8 @@ __global__ void __launch_bounds__(kStdSolveThreads) std_solve_kernel(StdConst c,
     for (int i = threadIdx.x; i <= n; i += blockDim.x) b.rhon[i] = 0.0;
     // the next markers' scales, from what the last ones recorded
     if (!c.fold) {
-      ScaleMaker<>(b.words, b.rec, n)
-          .make((unsigned *)sm, node_reach(__ldcg(b.vmax), c.reach), c.decay);
+      ScaleMaker<>(b.words, b.rec, b.storm, n)
+          .make((unsigned *)sm, node_reach(__ldcg(b.vmax), c.reach), c.decay, c.n_total);
       __syncthreads();
       if (threadIdx.x == 0) *b.vmax = 0u;
     }
@@ -290,7 +291,7 @@ __global__ void std_response_kernel(StdConst c, StdBufs b) {
 
 size_t std_smem(const StdConst &c, int copies) {
   return sizeof(double) * (size_t)(c.order + 1) * (1 + (size_t)copies) * c.n +
-         (c.fold ? 0 : sizeof(unsigned) * (c.n + 1));
+         (c.fold ? 0 : sizeof(unsigned) * (c.n + 2));
 }
 size_t std_solve_smem(const StdConst &c) { return sizeof(double) * 2 * (size_t)c.n; }
 

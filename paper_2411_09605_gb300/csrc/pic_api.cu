@@ -750,7 +750,7 @@ int init_es1d(pic_handle *h, const pic_species *species, const double *E0) {
   b.sd = nullptr;
   b.sds = nullptr;
   b.Jt = nullptr;
-  b.vmax = b.words = b.rec = nullptr;
+  b.vmax = b.words = b.rec = b.storm = nullptr;
   // a point's shape between the passes: its node and its offset (the moment
   // passes) or weights
   const size_t nsh = (size_t)(h->mom ? 1 : c.order + 1) * h->N;
@@ -765,6 +765,8 @@ int init_es1d(pic_handle *h, const pic_species *species, const double *E0) {
     // in one block, cleared together
     if ((rc = h->alloc(&b.Jt, mom_scalar_words(c)))) return rc;
     mom_scalars(c, b, b.Jt);
+    if ((rc = h->alloc(&b.storm, 4))) return rc;
+    CUDA_TRY(cudaMemsetAsync(b.storm, 0, sizeof(unsigned) * 4, h->st));
     CUDA_TRY(cudaMemsetAsync(b.Jt, 0, sizeof(double) * mom_scalar_words(c), h->st));
   }
   b.w = nullptr;
@@ -1211,6 +1213,8 @@ int init_std(pic_handle *h, const pic_species *species) {
       (rc = h->alloc(&b.err, 1)) || (rc = h->alloc(&h->ids, h->N)) ||
       (rc = h->alloc(&h->std_part, (size_t)h->lsd.grid * h->nsp + 1)))
     return rc;
+  if ((rc = h->alloc(&b.storm, 2))) return rc;
+  CUDA_TRY(cudaMemsetAsync(b.storm, 0, sizeof(unsigned) * 2, h->st));
   b.words = b.vmax + 1;   // cleared together
   b.rec = b.words + n + 1;
   h->b1.err = b.err;
@@ -1415,11 +1419,13 @@ int init_em1d(pic_handle *h, const pic_species *species, const double *E0, const
   // ESEC2, the next y* from pass E to pass C
   b.sd = b.sds = nullptr;
   b.si = b.sis = nullptr;
-  b.vmax = b.words = b.rec = nullptr;
+  b.vmax = b.words = b.rec = b.storm = nullptr;
   if (!h->mixed && ((rc = h->alloc(&b.sd, h->N)) || (rc = h->alloc(&b.si, h->N)) ||
                     (rc = h->alloc(&b.vmax, 2 + 8 * n))))
     return rc;
   if (b.vmax) {   // cleared together
+    if ((rc = h->alloc(&b.storm, 4))) return rc;
+    CUDA_TRY(cudaMemsetAsync(b.storm, 0, sizeof(unsigned) * 4, h->st));
     b.words = b.vmax + 2;
     b.rec = b.words + 4 * n;
   }
@@ -2418,6 +2424,7 @@ int grad_backward_mom(pic_handle *h, const double *Ebar, const double *xbar, con
   double *J2 = g.grid + 5 * nc;
   r.gtot = scal + mom_scalar_words(h->c1);
   r.tot = r.gtot + 1;
+  r.storm = h->b1.storm;
   r.umax = (unsigned *)(r.gtot + 5);
   r.mx = r.umax + 2;
   r.xb = mk;

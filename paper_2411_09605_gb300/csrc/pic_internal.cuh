@@ -261,6 +261,7 @@ struct Em1dBufs {
   int *sis;                  // -> pass C), as sd / si; null: formed again
   unsigned *words;           // [2][n][2] the nodes' scale words (fixed_moments.cuh) of J1, J2 and
   unsigned *rec;             // [2][n][2] the larger amounts recorded since
+  unsigned *storm;           // [2][2] outliers since, passes left that look around
   unsigned *vmax;            // [2] the largest |vy| (high word): of the last step, of this one
   double *E, *En;            // E^n, E^{n+1}: [2][n] (Ex, Ey); swapped after each step
   double *B, *Bn;            // Bz^n, Bz^{n+1}: [n]
@@ -313,6 +314,7 @@ struct StdBufs {
   double *resp;          // [n] E of a unit charge at node 0
   unsigned *words, *rec;    // [n + 1] the nodes' scale words (fixed_moments.cuh; several species,
                             // weights) and their range, [n] the larger charges recorded since
+  unsigned *storm;          // [2] outliers since, passes left that look around
   unsigned *vmax;           // [1] the largest |v| (high word)
   double *ke_part;       // [particle blocks]
   unsigned long long *fallback;
@@ -414,6 +416,8 @@ struct Es1dFp64Bufs {
   unsigned *words;          // and [2][nc + 1] the nodes' scale words (fixed_moments.cuh) of J1, J2
                             // and their range,
   unsigned *rec;            // [2][nc] the larger amounts recorded since
+  unsigned *storm;          // [2][2] outliers since, passes left that look around (kept when the
+                            // state is set anew)
   unsigned *vmax;           // and [2] the largest |v| (high word) by step parity
   double *E[2];             // ping-pong E^n / E^{n+1}
   double *J1[2];            // j^{n,*} (ESEC2), indexed by step parity
@@ -498,6 +502,7 @@ struct Es1dRevBufs {
   double *tot;              // [2][2] their totals
   unsigned *mx;             // [2][3][nc] exponents of the nodes' largest amounts
   unsigned *umax;           // [2] the largest |v*| (high word)
+  const unsigned *storm;    // the forward passes' (Es1dFp64Bufs)
   double *xb, *vb, *wb;     // [N] adjoints of the markers (x in cells)
   double *ub, *yb, *u, *ap, *dy;   // [N] marker scratch
   long long *D;

@@ -86,6 +86,25 @@ def test_heavy_marker_on_its_way(scheme, order):
 
 @pytest.mark.parametrize("order", [1, 2])
 @pytest.mark.parametrize("scheme", [1, 2])
+def test_fast_marker_among_slow_ones(scheme, order):
+    """One marker crosses a fifth of the domain in a step: the nodes that it does not
+    deposit to (its cells and their neighbours in every pass) hold the slow markers'
+    currents alone."""
+    rng = np.random.default_rng(6)
+    n, nc, L, dt, steps = 40_001, 400, 2 * np.pi, 0.01, 3
+    x, v = rng.uniform(0, L, n), SMALL * rng.standard_normal(n)
+    x[0], v[0] = 0.1013 * L, 0.2 * L / dt
+    prob = W.Problem1D("fast", L, nc, order, dt, 0, [W.Markers1D(-1.0, 1.0, x, v, None, 1e-9 * L / n)])
+    ref = oracle_run(prob, scheme, steps, remove_mean=False, E0=np.zeros(nc))["E"]
+    got = gpu_run(prob, scheme, steps, remove_mean=False, E0=np.zeros(nc))["E"]
+    there = (0.1013 + 0.1 * np.arange(2 * steps + 3)) * nc     # x^n and x^{n+1/2}
+    away = np.abs((np.arange(nc)[:, None] - there + nc / 2) % nc - nc / 2).min(axis=1) > 3
+    assert 0.0 < np.abs(ref[away]).max() < 1e-20
+    assert np.abs(got - ref)[away].max() <= 1e-11 * np.abs(ref[away]).max()
+
+
+@pytest.mark.parametrize("order", [1, 2])
+@pytest.mark.parametrize("scheme", [1, 2])
 @pytest.mark.parametrize("n,cells", [(30_001, 64), (30_001, 256)])
 def test_1d2v(n, cells, scheme, order):
     """Ey, whose update is the node's own jy (the oracle transforms it with the rest, so
